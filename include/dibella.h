@@ -140,9 +140,15 @@ int dibella_pack_reads(const char* ascii, const int64_t* ascii_offsets, int64_t 
  * per extension with an 8192-cell band in shared memory (the CTA form), and
  * beyond that by a warp whose band lives in the workspace (sized by
  * max_read_len: it cannot overflow).
+ * When a call passes no schedule (and the default is the built-in one), match
+ * 1, mismatch -1, gap -1 and 1 <= xdrop <= 59 take none of these but the
+ * bit-sliced form: 32 cells of a lane in one register per score bit, 1 to 32
+ * lanes per extension by the width of its band (a whole warp with 2 and 4
+ * words per lane for bands up to 4,096 cells, then the CTA form and the band in
+ * the workspace as above).
  * An extension is routed to narrow when xdrop <= narrow_max_xdrop and
  * min(remaining A, remaining B) <= narrow_max_len.  When a call passes no
- * schedule, batches with fewer than 1.5 extensions per resident narrow lane
+ * schedule and the bit-sliced form does not apply, batches with fewer than 1.5 extensions per resident narrow lane
  * go entirely to the wide form (they would wait on one lane's longest
  * extension), and for xdrop > 10 keys above 20000 (above 5000 in batches
  * with fewer than 7 extensions per lane) go to the wide form (a narrow lane
@@ -474,8 +480,9 @@ int dibella_autotune(const uint32_t* packed_words, const int64_t* read_word_offs
  * event and writes up to n_max phase durations in ms: queueing (expand, scan,
  * scatter), narrow form (first pass), second narrow pass (0 without one),
  * first wide launch, mid form (0 without one), the wide launch on the
- * escalations, the slot ladder with the CTA and global forms, combine;
- * returns the count written (8 after a batch).  Enable it before any capture
+ * escalations, the slot ladder with the CTA and global forms, combine (a
+ * batch in the bit-sliced form: its shared-lane launch stands as the narrow
+ * form, its whole-warp launch with the ladder); returns the count written (8 after a batch).  Enable it before any capture
  * (it creates the events). */
 int dibella_enable_phase_timing(int enable);
 int dibella_phase_times(float* ms_out, int n_max);
@@ -492,7 +499,9 @@ int dibella_phase_times(float* ms_out, int n_max);
  * extensions they handed on (restarted from the origin by the wider form or
  * the second narrow pass, so evaluated twice; not part of the cells of any
  * result), out[15] the extensions the first narrow pass handed to the
- * second.  Returns the number written (<= n_max, at most 16), or a negative
+ * second.  A batch in the bit-sliced form counts every extension as routed
+ * narrow, in out[2] the times one was suspended to be taken up again in other
+ * lanes, and its whole-warp launch with the ladder.  Returns the number written (<= n_max, at most 16), or a negative
  * status. */
 int dibella_batch_counters(const void* workspace, void* stream, int64_t* out, int n_max);
 

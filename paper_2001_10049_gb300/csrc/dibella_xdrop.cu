@@ -25,6 +25,10 @@
 //   global   one warp per extension with the band in workspace memory
 //   combine  seed + left + right, coordinates, cells; best seed per pair
 //
+// With unit scores, X <= 59 and no schedule given, the extensions instead run in
+// the bit-sliced form (xdrop_bits.cuh): one launch in which the warps deal their
+// lanes out to the extensions by the width of their bands.
+//
 // Arithmetic is int32 (limits on scores and read lengths in dibella.h keep
 // every value inside (-2^31, 2^31)); no tensor cores: this is not a dense
 // contraction.
@@ -80,7 +84,8 @@ enum { kQNarrow = 0, kQWide = 1, kQEsc1 = 2, kQLadder = 3, kQSmem = 7, kQGlobal 
 struct Counters {
   unsigned int tail[kNumQ];   // queue sizes (see the kQ* names)
   unsigned int head[kNumQ];   // pop cursors
-  unsigned int pad_[2];
+  unsigned int pool;          // words of the suspended extensions' pool handed out
+  unsigned int pad_;
   unsigned int bucket_count[2][DIBELLA_MAX_BUCKETS];
   unsigned int bucket_cursor[2][DIBELLA_MAX_BUCKETS];
   unsigned int stat[8];   // routed narrow, routed wide, escalated from narrow / wide /
@@ -118,6 +123,15 @@ struct ExtendParams {
   int cells_idx;  // Counters::cells entry the wide forms add to
   int narrow_cells_idx;  // Counters::cells entry of the one-lane forms (0 narrow, 6 mid)
   int narrow_esc_stat;   // Counters::stat entry counting their escalations (2 narrow, 6 mid)
+  int bits_esc_stat;     // Counters::stat entry counting the bit-sliced form's (2 narrow, 3 wide)
+  // Shared-lane bit-sliced form: lanes an extension counts for in its first
+  // `young` antidiagonals, and extensions that may share a warp.
+  int reserve, young, max_groups;
+  int* res_q;            // its suspended extensions, in the pool
+  int res_q_id;
+  long long res_cap;     // slots of res_q
+  uint32_t* pool;
+  unsigned pool_words;
   // Per-warp clock of one launch (null unless requested): warp w writes the
   // global timer (ns) when it starts, at [2w], and when it leaves, at [2w+1].
   unsigned long long* wclock;
@@ -1579,6 +1593,23 @@ __global__ void __launch_bounds__(NW * 32) narrow_kernel(ExtendParams p) {
   }
 }
 
+#include "xdrop_bits.cuh"
+
+// Bit-sliced form (see xdrop_bits.cuh).  Four blocks would fit an SM, two or one
+// are launched; asked for no residency, the compiler spilled to 72 registers.
+template <int NB>
+__global__ void __launch_bounds__(kBlockThreads, 4) bits_shared_kernel(ExtendParams p) {
+  __shared__ int map[kWarpsPerBlock][32];
+  warp_clock(p.wclock, 0);
+  bits_shared_run<NB>(p, map[threadIdx.x >> 5]);
+  warp_clock(p.wclock, 1);
+}
+
+template <int NB, int W>
+__global__ void __launch_bounds__(kBlockThreads) bits_warp_kernel(ExtendParams p) {
+  bits_warp_run<NB, W>(p);
+}
+
 // Global-band form: one warp per extension, band in workspace memory.
 __global__ void __launch_bounds__(kBlockThreads) global_kernel(ExtendParams p) {
   const int gwarp = (blockIdx.x * kBlockThreads + threadIdx.x) >> 5;
@@ -1839,12 +1870,14 @@ __global__ void __launch_bounds__(32) per_pair_kernel(const uint32_t* __restrict
 thread_local std::string g_last_error;
 
 std::mutex g_mu;
-dibella_schedule_t g_default_schedule = {
+constexpr dibella_schedule_t kDefaultSchedule = {
     /*narrow_max_xdrop=*/30, /*narrow_max_len=*/1 << 30, /*narrow_band_cap=*/48,
     /*wide_slots=*/0, /*wide_packed=*/1, /*wide_group_lanes=*/0, /*wide_blocks_per_sm=*/0,
     /*narrow_blocks_per_sm=*/0,
     /*n_buckets=*/6, {500, 2000, 5000, 10000, 20000, 0, 0, 0}, /*mid_band_cap=*/0, /*narrow_split_d=*/0,
     /*narrow_unroll=*/0, /*narrow_track=*/1};
+dibella_schedule_t g_default_schedule = kDefaultSchedule;
+bool g_own_default = false;  // dibella_set_default_schedule gave another one: it is followed as given
 
 struct DeviceInfo {
   bool ready = false;
@@ -1859,6 +1892,20 @@ struct DeviceInfo {
 };
 std::mutex g_dev_mu;
 DeviceInfo g_dev[64];
+
+// The bit-sliced form by the planes that X needs (kD = 2^planes - 2 has to stay
+// above every live value: X <= 2^planes - 5).  Each plane more costs about 9% of
+// an antidiagonal (107 warp instructions at 5 planes).  Beyond X = 59 the int16
+// forms run: a seventh plane would take X to 123, where no workload goes.
+using BitsKernel = void (*)(ExtendParams);
+struct BitsForms {
+  int max_x;
+  BitsKernel shared, warp;
+};
+const BitsForms kBitsForms[3] = {{11, bits_shared_kernel<4>, bits_warp_kernel<4, 4>},
+                                 {27, bits_shared_kernel<5>, bits_warp_kernel<5, 4>},
+                                 {59, bits_shared_kernel<6>, bits_warp_kernel<6, 4>}};
+constexpr int kBitsMaxX = 59;
 
 bool g_timing = false;
 cudaEvent_t g_ev[10] = {};
@@ -2186,6 +2233,27 @@ cudaError_t launch_wide(const DeviceInfo& D, const dibella_schedule_t& sch_in, i
   return cudaGetLastError();
 }
 
+// The forms for the widest bands: the CTA form on Smem (outgrown -> Global),
+// the global form on Global; then phase event 7.
+int launch_widest(const DeviceInfo& D, ExtendParams ep, int* const q[kNumQ], cudaStream_t st) {
+  cudaError_t e;
+  ep.wide_q = q[kQSmem];
+  ep.wide_q_id = kQSmem;
+  ep.esc_q = q[kQGlobal];
+  ep.esc_q_id = kQGlobal;
+  wide_cta_kernel<<<D.sms * D.cta_blocks, kCtaThreads, kCtaSmemBytes, st>>>(ep);
+  ++g_launches;
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "wide_cta launch");
+
+  ep.wide_q = q[kQGlobal];
+  ep.wide_q_id = kQGlobal;
+  global_kernel<<<kGlobalWarps / kWarpsPerBlock, kBlockThreads, 0, st>>>(ep);
+  ++g_launches;
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "global launch");
+  record(st, 7);
+  return DIBELLA_OK;
+}
+
 // All extension launches of one batch, in stream order:
 //   narrow form        on Narrow        (outgrown -> Esc1)
 //   wide form (S slots) on Wide         (outgrown -> ladder queue of S)
@@ -2309,22 +2377,66 @@ int launch_extensions(const DeviceInfo& D, const dibella_schedule_t& sch_in, int
     cur_q = next_q;
   }
   ep.forward_max = 0;
+  return launch_widest(D, ep, q, st);
+}
 
-  ep.wide_q = q[kQSmem];
-  ep.wide_q_id = kQSmem;
-  ep.esc_q = q[kQGlobal];
-  ep.esc_q_id = kQGlobal;
-  wide_cta_kernel<<<D.sms * D.cta_blocks, kCtaThreads, kCtaSmemBytes, st>>>(ep);
-  ++g_launches;
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "wide_cta launch");
+// All extension launches of a batch in the bit-sliced form, in stream order:
+//   shared-lane form on Narrow  (every extension; suspended ones go through the
+//                               resume queue, which lies over the ladder's
+//                               queues, and come back within the launch)
+//   whole-warp form on Ladder   (bands beyond 2,048 cells)
+//   CTA form on Smem, global form on Global, as in launch_extensions
+// Phase events: 2 to 6 after the shared-lane launch, 7 after the others.
+int launch_extensions_bits(const DeviceInfo& D, long long n_ext, ExtendParams ep, int* const q[kNumQ],
+                           cudaStream_t st) {
+  cudaError_t e;
+  const int X = ep.sc.X;
+  const BitsForms& F = kBitsForms[X <= kBitsForms[0].max_x ? 0 : (X <= kBitsForms[1].max_x ? 1 : 2)];
+  // Lanes to count on: unrelated sequences settle at a band of about 5.3 X cells
+  // (132 at X = 25), plus the margins.  Measured around this rule (ms, lanes
+  // 3/4, 4/5, 5/6, 9/10 at X = 7, 15, 25, 50): 28.3/29.9, 41.6/44.5, 58.2/55.3, 47.2/49.3.
+  ep.reserve = std::max(kInitLanes, (5 * X + 67) / 32);
+  ep.young = 20 * X;
+  // Warps per SM: the loop keeps the integer pipe 75% busy with one warp per
+  // scheduler and about 95% with two; more only make each extension slower, and
+  // the longest one ends the launch (E. coli-sized reads at X = 25, 300,000
+  // extensions: 70 / 55 / 74 ms with 1 / 2 / 3 blocks).  Small batches take one,
+  // and spread out over all warps: each extension runs fastest alone.
+  const long long lanes = 32ll * kWarpsPerBlock * D.sms;
+  const int blocks = n_ext * ep.reserve >= 8 * lanes ? 2 : 1;
+  const long long warps = (long long)D.sms * blocks * kWarpsPerBlock;
+  ep.max_groups = (int)std::min<long long>(16, std::max<long long>(1, (n_ext + warps - 1) / warps));
+  ep.res_q = q[kQLadder + 1];
+  ep.res_q_id = kQLadder + 1;
+  ep.res_cap = q[kQSmem] - q[kQLadder + 1];
+  ep.pool = (uint32_t*)ep.gband;  // free until the global form runs
+  ep.pool_words = (unsigned)std::min<long long>(3ll * ep.gcap * kGlobalWarps, 1ll << 31);
+  if ((e = cudaMemsetAsync(ep.res_q, 0xFF, sizeof(int) * (size_t)ep.res_cap, st)) != cudaSuccess)
+    return cuda_fail(e, "cudaMemsetAsync");
 
-  ep.wide_q = q[kQGlobal];
-  ep.wide_q_id = kQGlobal;
-  global_kernel<<<kGlobalWarps / kWarpsPerBlock, kBlockThreads, 0, st>>>(ep);
+  ep.wide_q = q[kQNarrow];
+  ep.wide_q_id = kQNarrow;
+  ep.esc_q = q[kQLadder];
+  ep.esc_q_id = kQLadder;
+  ep.cells_idx = 0;
+  ep.bits_esc_stat = 2;
+  ep.wclock = clock_for(1, (int)warps, st);
+  F.shared<<<D.sms * blocks, kBlockThreads, 0, st>>>(ep);
   ++g_launches;
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "global launch");
-  record(st, 7);
-  return DIBELLA_OK;
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "bit-sliced launch");
+  ep.wclock = nullptr;
+  for (int i = 2; i <= 6; ++i) record(st, i);
+
+  ep.wide_q = q[kQLadder];
+  ep.wide_q_id = kQLadder;
+  ep.esc_q = q[kQSmem];
+  ep.esc_q_id = kQSmem;
+  ep.cells_idx = 5;
+  ep.bits_esc_stat = 3;
+  F.warp<<<D.sms, kBlockThreads, 0, st>>>(ep);
+  ++g_launches;
+  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "bit-sliced whole-warp launch");
+  return launch_widest(D, ep, q, st);
 }
 
 int expand_and_queue(const uint32_t* words, const int64_t* offs, const int32_t* lens, int64_t n_reads,
@@ -2425,6 +2537,7 @@ int dibella_set_default_schedule(const dibella_schedule_t* sched) {
   if (!sched || validate_schedule(*sched) != DIBELLA_OK) return DIBELLA_EINVAL;
   std::lock_guard<std::mutex> lk(g_mu);
   g_default_schedule = *sched;
+  g_own_default = memcmp(sched, &kDefaultSchedule, sizeof(kDefaultSchedule)) != 0;
   return DIBELLA_OK;
 }
 
@@ -2447,11 +2560,14 @@ int dibella_xdrop_batch(const uint32_t* packed_words, const int64_t* read_word_o
     return DIBELLA_EINVAL;
   if (!workspace || ((uintptr_t)workspace & 255)) return DIBELLA_EINVAL;
   dibella_schedule_t sch;
+  bool own_default = false;
   if (sched) {
     if (validate_schedule(*sched) != DIBELLA_OK) return DIBELLA_EINVAL;
     sch = *sched;
   } else {
-    dibella_get_default_schedule(&sch);
+    std::lock_guard<std::mutex> lk(g_mu);
+    sch = g_default_schedule;
+    own_default = g_own_default;
   }
   const int gcap = gcap_from_workspace(n_pairs, workspace_bytes);
   if (gcap < 64) return DIBELLA_ENOMEM;
@@ -2472,7 +2588,15 @@ int dibella_xdrop_batch(const uint32_t* packed_words, const int64_t* read_word_o
   // keys above 20000 (above 5000 unless the batch gives each lane 7 or more
   // extensions) go straight to the wide form.  An explicit schedule is
   // followed as given.
-  if (sched == nullptr) {
+  // Without a schedule, unit scores (every named workload's) at X from 1 to 59
+  // take the bit-sliced form: it packs the lanes itself, so every extension goes
+  // to its one queue, longest first.
+  const bool bits = sched == nullptr && !own_default && scoring.match == 1 && scoring.mismatch == -1 &&
+                    scoring.gap == -1 && scoring.xdrop >= 1 && scoring.xdrop <= kBitsMaxX;
+  if (bits) {
+    sch.narrow_max_xdrop = INT32_MAX;
+    sch.narrow_max_len = INT32_MAX;
+  } else if (sched == nullptr) {
     const int wt = sch.narrow_band_cap;
     const long long narrow_lanes =
         (long long)D->sms *
@@ -2509,7 +2633,7 @@ int dibella_xdrop_batch(const uint32_t* packed_words, const int64_t* read_word_o
   ep.long_q = nullptr;
   int* q[kNumQ];
   for (int i = 0; i < kNumQ; ++i) q[i] = (int*)(ws + L.queue[i]);
-  rc = launch_extensions(*D, sch, scoring.xdrop, ep, q, st);
+  rc = bits ? launch_extensions_bits(*D, 2 * n_pairs, ep, q, st) : launch_extensions(*D, sch, scoring.xdrop, ep, q, st);
   if (rc != DIBELLA_OK) return rc;
   rc = finish(read_lengths, pairs, n_pairs, k, results, ep.ext, st);
   record(st, 8);
