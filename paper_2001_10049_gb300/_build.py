@@ -16,7 +16,8 @@ LIB_DEBUG = os.path.join(HERE, "libdibella_debug.so")
 SOURCES = [os.path.join(CSRC, "dibella_xdrop.cu"), os.path.join(CSRC, "dibella_kmers.cu"),
            os.path.join(CSRC, "dibella_traceback.cu"), os.path.join(CSRC, "dibella_peak.cu"),
            os.path.join(CSRC, "dibella_pack.cpp")]
-HEADERS = [os.path.join(INCLUDE, "dibella.h"), os.path.join(CSRC, "xdrop_bits.cuh")]
+HEADERS = [os.path.join(INCLUDE, "dibella.h"), os.path.join(CSRC, "xdrop_bits.cuh"),
+           os.path.join(CSRC, "xdrop_bits_run.cuh")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 _lock = threading.Lock()
 

@@ -17,6 +17,19 @@
 // (the band's first i and its width), the band's moves at 2 bits per cell
 // (packed by warp reductions), and a trailer word (the width again), so that
 // lane 0 can walk back one antidiagonal at a time from the best cell.
+//
+// With unit scores and X <= 59 the extension runs in the bit-sliced form
+// (xdrop_bits.cuh) with one word of cells a lane: the comparisons that choose a
+// cell's value are its move, two planes of 32 cells a lane, so recording costs a
+// store and a few counts.  Both extensions run at once, 16 lanes each, where
+// their bands and move words allow.  The walk back is done by the lanes
+// together: each holds the move words of one or two of the next 32
+// antidiagonals, and a run of diagonal steps is one look-up.  Bands beyond 990
+// cells take the general form above.
+// 2,000 accepted overlaps of E. coli-sized reads at X = 25 take 16.0 to 19.7 ms
+// (the general form, bound by its rows in memory and one lane's walk, 52 to 73):
+// now the longest overlap alone (69,700 antidiagonals, 14.8 ms, about a third
+// of it the walk), which is a serial chain.
 
 #include <cuda_runtime.h>
 
@@ -25,6 +38,11 @@
 #include "../../include/dibella.h"
 
 namespace {
+
+constexpr unsigned kFull = 0xFFFFFFFFu;
+__device__ __forceinline__ uint32_t ldg_word(const uint32_t* __restrict__ words, long long w) { return __ldg(words + w); }
+
+#include "xdrop_bits.cuh"
 
 constexpr int kTbThreads = 128;
 constexpr int32_t kDead = INT32_MIN / 2;  // dead, or outside its antidiagonal's band
@@ -257,10 +275,429 @@ __host__ __device__ bool tb_walk(const TbArgs& p, const TbSeq& s, const TbExt& e
   return true;
 }
 
+// ---- bit-sliced form ---------------------------------------------------------
+// Its slot: a word for each antidiagonal (lanes that hold its band | place of
+// the first one's lowest cell / 32, see below), where the general form has its
+// rows, and the move words: two (hi, lo) of each such lane, antidiagonal after
+// antidiagonal.  Those take no more words than the general form's records
+// (2 T <= 3 + ceil(width / 16) for a band of any width over T words), so what
+// fits is decided by the general form's count.  The window moves by whole words,
+// so that the lowest cell of a lane's word is i = (d + 1) / 2 + 32 q.
+constexpr int kTbWin = 1024;
+
+struct TbBits {
+  int best, i_end, j_end;
+  long long cells;
+  long long best_off;  // the best antidiagonal's first move word
+  bool recorded;       // every antidiagonal up to the best one fit
+};
+
+// The extension of a (ascending from a0) and b (descending from b0) by the
+// whole warp; false if its band outgrew the window.
+template <int NB>
+__device__ bool tb_extend_bits(const TbArgs& p, long long a0, long long b0, int m, int n, const uint32_t (&kx)[NB],
+                               const uint32_t (&ky)[NB], uint32_t* head, uint32_t* moves, TbBits& e) {
+  using F = BitForm<NB, 1>;
+  constexpr int kMargin = 17;  // 32 antidiagonals between looks: at most 16 places either way
+  const int lane = threadIdx.x & 31;
+  const GroupMasks gm = group_masks(lane, 0, 32);
+  typename F::Lane L;
+  F::clear(L);
+  F::init(L, kTbWin / 2 - 32 * lane);
+  int f0 = -kTbWin / 2;
+  long long off = 0, used = 0, imp_off = 0;
+  bool keep = true, imp_keep = true;
+  e.i_end = e.j_end = 0;
+  e.cells = 0;
+  auto record = [&](const BitMoves<1>& mv) {
+    const unsigned bal = __ballot_sync(kFull, mv.band[0] != 0);
+    if (bal == 0) return;
+    const int width = __reduce_add_sync(kFull, __popc(mv.band[0]));
+    const int t = __popc(bal), first = __ffs((int)bal) - 1;
+    e.cells += width;
+    const int rec = 3 + ((width + 15) >> 4);
+    keep = keep && used + rec <= p.moves_words;
+    if (L.imp_d == L.d) {
+      imp_off = off;
+      imp_keep = keep;
+    }
+    if (!keep) return;
+    used += rec;
+    if (lane == 0) head[L.d] = (uint32_t)t | ((uint32_t)((f0 >> 5) + first) << 6);
+    if (mv.band[0] != 0) *(uint2*)(moves + off + 2 * (lane - first)) = make_uint2(mv.hi[0], mv.lo[0]);
+    off += 2 * t;
+  };
+  F::load_window(L, p.words, a0, b0, m, n, f0 + 32 * lane, 0);
+  for (;;) {
+    F::load_feed(L, p.words, a0, b0, m, n, f0 + ((L.d + 1) >> 1) + 32 * lane, L.d);
+#pragma unroll 1
+    for (int k = 0; k < 32; k += 2) {
+      BitMoves<1> mv;
+      F::template step<true>(L, L.r[0], L.r[1], kx, ky, gm, &mv);
+      record(mv);
+      F::template step<false>(L, L.r[1], L.r[0], kx, ky, gm, &mv);
+      record(mv);
+    }
+    const uint32_t live[1] = {~L.dead[0]};
+    int lo, hi;
+    group_ends<1>(live, lane, 0, kFull, lo, hi);
+    if (lo >= kMargin && hi <= kTbWin - 1 - kMargin) continue;
+    int at, at_hi;
+    group_ends<1>(L.imp, lane, 0, kFull, at, at_hi);
+    if (L.imp_d >= 0) {
+      e.i_end = f0 + ((L.imp_d + 1) >> 1) + at;
+      e.j_end = L.imp_d - e.i_end;
+    }
+    L.imp_d = -1;
+    if (lo < 0) break;
+    const int by = ((lo + hi) / 2 - kTbWin / 2 + (lo < kMargin ? -16 : 16)) / 32;
+    if (lo - 32 * by < kMargin || hi - 32 * by > kTbWin - 1 - kMargin) return false;
+    const int src = lane + by;
+    const bool held = src >= 0 && src < 32;
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+      const uint32_t x = __shfl_sync(kFull, L.r[0][0][k], src & 31), y = __shfl_sync(kFull, L.r[1][0][k], src & 31);
+      L.r[0][0][k] = held ? x : F::dead_plane(k);
+      L.r[1][0][k] = held ? y : F::dead_plane(k);
+    }
+    const uint32_t dd = __shfl_sync(kFull, L.dead[0], src & 31);
+    L.dead[0] = held ? dd : 0xFFFFFFFFu;
+    f0 += 32 * by;
+    F::load_window(L, p.words, a0, b0, m, n, f0 + ((L.d + 1) >> 1) + 32 * lane, L.d);
+  }
+  e.best = L.best;
+  e.best_off = imp_off;
+  e.recorded = imp_keep;
+  __syncwarp();  // the records are read by other lanes
+  return true;
+}
+
+// A run-length writer whose state all lanes of a group hold; its first lane
+// writes, run x to out[step * x].
+struct TbWarpRuns {
+  uint32_t* out;
+  long long cap;
+  int step;
+  bool writer;
+  int n;
+  uint32_t op, len;
+  __device__ void push(uint32_t o, uint32_t l) {
+    if (len && o == op) {
+      len += l;
+      return;
+    }
+    flush();
+    op = o;
+    len = l;
+  }
+  __device__ void flush() {
+    if (!len) return;
+    if (writer && n < cap) out[(long long)step * n] = (len << 4) | op;
+    ++n;
+    len = 0;
+  }
+};
+
+// The columns from cell (i, j), whose antidiagonal's move words start at off,
+// back to the origin.  A group is G lanes (16: two walks at once, or 32); lane l
+// of it takes the antidiagonals d - l (and d - l - 16) of the next 32 and loads
+// the two words that the path can meet there, so that a column is a look-up of
+// every lane and one shuffle.  The words of a downward stream lie below `moves`.
+template <int G>
+__device__ void tb_walk_bits(const uint32_t* head, const uint32_t* moves, bool down, int i, int j, long long off,
+                             TbWarpRuns& runs) {
+  constexpr int U = 32 / G;
+  const int gl = threadIdx.x & (G - 1);
+  int d = i + j;
+  while (__any_sync(kFull, d > 0)) {
+    const int d0 = d;
+    int i0[U], w[U], before = 0;
+    long long mine[U];
+    uint2 top[U], low[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int dl = d - gl - G * u;
+      const uint32_t h = dl >= 1 ? head[dl] : 0u;
+      const int t = (int)(h & 63u);
+      int s = t;  // words of the antidiagonals from d down to this one
+#pragma unroll
+      for (int o = 1; o < G; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, s, o, G);
+        if (gl >= o) s += v;
+      }
+      s += before;
+      before = __shfl_sync(kFull, s, G - 1, G);
+      if (u == 0) off += 2 * __shfl_sync(kFull, t, 0, G);
+      mine[u] = off - 2ll * s;
+      i0[u] = ((dl + 1) >> 1) + 32 * ((int)h >> 6);
+      w[u] = (i - i0[u]) >> 5;  // the path meets [i - 31, i]: words w and w - 1
+      const uint2 zero = make_uint2(0, 0);
+      const long long at = mine[u] + 2 * w[u];
+      top[u] = w[u] >= 0 && w[u] < t ? *(const uint2*)(moves + (down ? -2 - at : at)) : zero;
+      low[u] = w[u] >= 1 && w[u] - 1 < t ? *(const uint2*)(moves + (down ? -at : at - 2)) : zero;
+    }
+    // From the present cell (antidiagonal d0 - x) every lane looks up the move of
+    // the cell that a run of diagonal steps would reach on its antidiagonal (the
+    // diagonal keeps to every other one): the lowest of them with another move
+    // ends the run, and that move follows it.
+    while (__any_sync(kFull, d > 0 && d > d0 - 30)) {
+      const int x = d0 - d;
+      uint32_t gap = 0, eq = 0;  // bit l: antidiagonal d0 - l
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int pos = i - ((gl + G * u - x) >> 1) - i0[u];
+        const bool at_top = (pos >> 5) == w[u];
+        const uint32_t hi = at_top ? top[u].x : low[u].x, lo = at_top ? top[u].y : low[u].y;
+        const unsigned bh = __ballot_sync(kFull, (hi >> (pos & 31)) & 1u), bl = __ballot_sync(kFull, (lo >> (pos & 31)) & 1u);
+        if (G == 32) {
+          gap = bh;
+          eq = bl;
+        } else {
+          gap |= ((bh >> (threadIdx.x & 16)) & 0xFFFFu) << (G * u);
+          eq |= ((bl >> (threadIdx.x & 16)) & 0xFFFFu) << (G * u);
+        }
+      }
+      if (d > 0 && d > d0 - 30) {
+        const int stop = min(30 + (x & 1), d0);
+        const uint32_t ends = gap & (0x55555555u << (x & 1)) & (0xFFFFFFFFu << x);
+        const int at = ends ? __ffs((int)ends) - 1 : 32;
+        int r = (min(at, stop) - x) >> 1;  // diagonal steps
+        i -= r;
+        j -= r;
+        uint32_t same = (eq >> x) & 0x55555555u;
+        while (r > 0) {
+          const bool is = same & 1u;
+          const uint32_t other = is ? ~same & 0x55555555u : same;
+          const int c = min(r, other ? (__ffs((int)other) - 1) >> 1 : 16);
+          runs.push(is ? kOpEq : kOpX, (uint32_t)c);
+          same = shr_clamp(same, 2u * (uint32_t)c);
+          r -= c;
+        }
+        if (at < stop) {
+          const bool in_b = (eq >> at) & 1u;
+          runs.push(in_b ? kOpIns : kOpDel, 1);
+          i -= !in_b;
+          j -= in_b;
+        }
+        d = i + j;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long v = __shfl_sync(kFull, mine[u], (d0 - d) & (G - 1), G);
+      off = (d0 - d) / G == u ? v : off;
+    }
+  }
+}
+
+// Left (lanes 0-15) and right extension (lanes 16-31) of a seed at once, 16
+// words of cells each: both share the slot, the left one's move words growing up
+// from `moves`, the right one's down from `end`, and head (the right one's
+// antidiagonals after the left one's).  Whether everything fits is decided on an
+// upper bound of the general form's count; false if that or a window does not do
+// (the caller then takes the extensions one after the other).
+template <int NB>
+__device__ bool tb_extend_both(const TbArgs& p, long long a0, long long b0, int m, int n, const uint32_t (&kx)[NB],
+                               const uint32_t (&ky)[NB], uint32_t* head, uint32_t* moves, uint32_t* end, TbBits& e) {
+  using F = BitForm<NB, 1>;
+  constexpr int kMargin = 17, kWin = 512;
+  const int lane = threadIdx.x & 31, first = lane & 16, gl = lane & 15;
+  const bool down = first != 0;
+  const GroupMasks gm = group_masks(lane, first, 16);
+  typename F::Lane L;
+  F::clear(L);
+  F::init(L, kWin / 2 - 32 * gl);
+  int f0 = -kWin / 2;
+  int off = 0, imp_off = 0;
+  e.i_end = e.j_end = 0;
+  uint2* const base = (uint2*)(down ? end - 2 : moves);
+  const long long room = end - moves < (1ll << 30) ? end - moves : (1ll << 30);
+  auto record = [&](const BitMoves<1>& mv) {
+    const unsigned bal = __ballot_sync(kFull, mv.band[0] != 0) & gm.grp;
+    const int t = __popc(bal), at = __ffs((int)bal) - 1;
+    imp_off = L.imp_d == L.d ? off : imp_off;
+    if (bal && gl == 0) head[L.d] = (uint32_t)t | ((uint32_t)((f0 >> 5) + at - first) << 6);
+    const int o = off + lane - at;
+    if (mv.band[0] != 0) base[down ? -o : o] = make_uint2(mv.hi[0], mv.lo[0]);
+    off += t;
+  };
+  F::load_window(L, p.words, a0, b0, m, n, f0 + 32 * gl, 0);
+  for (;;) {
+    // Room for 32 antidiagonals of 16 words on both sides.
+    const int other = __shfl_xor_sync(kFull, off, 16);
+    if (__any_sync(kFull, 2ll * (off + other + 2 * 32 * 16) > room ||
+                              2ll * (off + 32 * 16) + 3ll * (L.d + 32) > p.moves_words))
+      return false;
+    F::load_feed(L, p.words, a0, b0, m, n, f0 + ((L.d + 1) >> 1) + 32 * gl, L.d);
+#pragma unroll 1
+    for (int k = 0; k < 32; k += 2) {
+      BitMoves<1> mv;
+      F::template step<true>(L, L.r[0], L.r[1], kx, ky, gm, &mv);
+      record(mv);
+      F::template step<false>(L, L.r[1], L.r[0], kx, ky, gm, &mv);
+      record(mv);
+    }
+    const uint32_t live[1] = {~L.dead[0]};
+    int lo, hi;
+    group_ends<1>(live, lane, first, gm.grp, lo, hi);
+    const bool done = lo < 0, near_end = !done && (lo < kMargin || hi > kWin - 1 - kMargin);
+    if (__any_sync(kFull, near_end) || __all_sync(kFull, done)) {
+      int at, at_hi;
+      group_ends<1>(L.imp, lane, first, gm.grp, at, at_hi);
+      if (L.imp_d >= 0) {
+        e.i_end = f0 + ((L.imp_d + 1) >> 1) + at;
+        e.j_end = L.imp_d - e.i_end;
+      }
+      L.imp_d = -1;
+      L.imp[0] = 0;
+      if (__all_sync(kFull, done)) break;
+      const int by = near_end ? ((lo + hi) / 2 - kWin / 2 + (lo < kMargin ? -16 : 16)) / 32 : 0;
+      if (__any_sync(kFull, near_end && (lo - 32 * by < kMargin || hi - 32 * by > kWin - 1 - kMargin))) return false;
+      const int src = gl + by;
+      const bool held = src >= 0 && src < 16;
+#pragma unroll
+      for (int k = 0; k < NB; ++k) {
+        const uint32_t x = __shfl_sync(kFull, L.r[0][0][k], src & 15, 16), y = __shfl_sync(kFull, L.r[1][0][k], src & 15, 16);
+        L.r[0][0][k] = held ? x : F::dead_plane(k);
+        L.r[1][0][k] = held ? y : F::dead_plane(k);
+      }
+      const uint32_t dd = __shfl_sync(kFull, L.dead[0], src & 15, 16);
+      L.dead[0] = held ? dd : 0xFFFFFFFFu;
+      f0 += 32 * by;
+      F::load_window(L, p.words, a0, b0, m, n, f0 + ((L.d + 1) >> 1) + 32 * gl, L.d);
+    }
+  }
+  long long cells = L.cells;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) cells += __shfl_xor_sync(kFull, cells, o);
+  e.cells = cells;
+  e.best = L.best;
+  e.best_off = 2ll * imp_off;
+  e.recorded = true;
+  __syncwarp();  // the records are read by other lanes
+  return true;
+}
+
+__device__ __forceinline__ TbBits tb_from_lane(const TbBits& e, int lane) {
+  TbBits r;
+  r.best = __shfl_sync(kFull, e.best, lane);
+  r.i_end = __shfl_sync(kFull, e.i_end, lane);
+  r.j_end = __shfl_sync(kFull, e.j_end, lane);
+  r.cells = __shfl_sync(kFull, e.cells, lane);
+  r.best_off = __shfl_sync(kFull, e.best_off, lane);
+  r.recorded = true;
+  return r;
+}
+
+// Seed t as tb_seed does it, in the bit-sliced form; false (results to be
+// written by tb_seed) if a band outgrew its window.  The seed is valid.
+template <int NB>
+__device__ bool tb_seed_bits(const TbArgs& p, long long t, char* scratch, const dibella_pair_t& pr, long long lenA,
+                             long long lenB) {
+  const int lane = threadIdx.x & 31;
+  const int k = p.k;
+  uint32_t kx[NB], ky[NB];
+  bits_threshold<NB>(p.X, kx, ky);
+  uint32_t* head = (uint32_t*)scratch;
+  uint32_t* moves = head + ((2ll * p.max_len + 5) & ~1ll);
+  const long long fA = p.word_offsets[pr.read_a] * 16, rA = fA + tb_copy_words(lenA) * 16;
+  const long long fB = p.word_offsets[pr.read_b] * 16, rB = fB + tb_copy_words(lenB) * 16;
+  const long long bp0 = pr.strand ? rB : fB;  // B', and its reverse complement
+  const long long bc0 = pr.strand ? fB : rB;
+  const long long pa = pr.pos_a;
+  const long long pb = pr.strand ? lenB - pr.pos_b - k : (long long)pr.pos_b;
+  const bool eq = lane < k && tb_base(p.words, fA, pa + lane) == tb_base(p.words, bp0, pb + lane);
+  const unsigned seed_eq = __ballot_sync(kFull, eq);
+  const int n_eq = __popc(seed_eq);
+  // Left: a(x) = A[pa-1-x] from A's reverse complement, b(y) = B'[pb-1-y];
+  // right: a(x) = A[pa+k+x], b(y) = B'[pb+k+y] from the other copy.
+  const long long la = rA + (lenA - pa), lb = bp0 + pb - 1, ra = fA + pa + k, rb = bc0 + (lenB - 1 - pb - k);
+  const int lm = (int)pa, ln = (int)pb, rm = (int)(lenA - pa - k), rn = (int)(lenB - pb - k);
+  uint32_t* ops = p.ops + t * (long long)p.ops_per_seed;
+  TbWarpRuns runs{ops, p.ops_per_seed, 1, lane == 0, 0, 0, 0};
+  TbWarpRuns back{nullptr, 0, -1, lane == 0, 0, 0, 0};
+  const uint32_t* back_last = nullptr;  // the right walk's last run; the others follow it, last to first
+  TbBits el, er;
+  bool ok = true;
+  auto seed_columns = [&]() {
+    for (int q = 0; q < k; ++q) runs.push((seed_eq >> q) & 1u ? kOpEq : kOpX, 1);
+  };
+  // The walk of the right extension writes its run x to its head[d - x], an
+  // antidiagonal that it has left (a run is a column at least).
+  const bool rt = lane >= 16;
+  TbBits e;
+  uint32_t* own = head + (rt ? lm + ln + 1 : 0);
+  uint32_t* end = (uint32_t*)(scratch + 12ll * (p.max_len + 2) + 4 * p.moves_words);
+  end -= (end - head) & 1;
+  if (tb_extend_both<NB>(p, rt ? ra : la, rt ? rb : lb, rt ? rm : lm, rt ? rn : ln, kx, ky, own, moves, end, e)) {
+    const int d = e.i_end + e.j_end;
+    TbWarpRuns both{rt ? own + d : ops, rt ? (long long)d : (long long)p.ops_per_seed, rt ? -1 : 1, (lane & 15) == 0,
+                    0, 0, 0};
+    tb_walk_bits<16>(own, rt ? end : moves, rt, e.i_end, e.j_end, e.best_off, both);
+    if (rt) both.flush();
+    __syncwarp();
+    el = tb_from_lane(e, 0);
+    er = tb_from_lane(e, 16);
+    runs.n = __shfl_sync(kFull, both.n, 0);
+    runs.op = __shfl_sync(kFull, both.op, 0);
+    runs.len = __shfl_sync(kFull, both.len, 0);
+    back.n = __shfl_sync(kFull, both.n, 16);
+    back_last = head + (lm + ln + 1) + er.i_end + er.j_end - back.n + 1;
+    seed_columns();
+  } else {
+    if (!tb_extend_bits<NB>(p, la, lb, lm, ln, kx, ky, head, moves, el)) return false;
+    ok = el.recorded;
+    if (ok) {
+      tb_walk_bits<32>(head, moves, false, el.i_end, el.j_end, el.best_off, runs);
+      seed_columns();
+    }
+    __syncwarp();  // the left walk has read the records before the right extension rewrites them
+    if (!tb_extend_bits<NB>(p, ra, rb, rm, rn, kx, ky, head, moves, er)) return false;
+    if (ok) ok = er.recorded;
+    if (ok) {
+      const int d = er.i_end + er.j_end;
+      back.out = head + d;
+      back.cap = d;
+      tb_walk_bits<32>(head, moves, false, er.i_end, er.j_end, er.best_off, back);
+      back.flush();
+      __syncwarp();
+      back_last = head + d - back.n + 1;
+    }
+  }
+  if (back.n > 0) {  // the first may join the seed's last run; the others follow as they are
+    const uint32_t w = back_last[0];
+    runs.push(w & 15u, w >> 4);
+    runs.flush();
+    for (int x = lane; x < back.n - 1; x += 32)
+      if (runs.n + x < runs.cap) runs.out[runs.n + x] = back_last[1 + x];
+    runs.n += back.n - 1;
+  }
+  runs.flush();
+  if (lane == 0) {
+    dibella_result_t r;
+    r.score_left = el.best;
+    r.score_right = er.best;
+    r.score = n_eq * p.M + (k - n_eq) * p.S + el.best + er.best;
+    r.begin_a = (uint32_t)(pa - el.i_end);
+    r.end_a = (uint32_t)(pa + k + er.i_end);
+    const long long bb = pb - el.j_end, eb = pb + k + er.j_end;
+    r.begin_b = (uint32_t)(pr.strand ? lenB - eb : bb);
+    r.end_b = (uint32_t)(pr.strand ? lenB - bb : eb);
+    r.status = n_eq == k ? 0 : DIBELLA_RES_SEED_MISMATCH;
+    r.cells = el.cells + er.cells;
+    p.results[t] = r;
+    p.n_ops[t] = !ok ? -2 : (runs.n > runs.cap ? -1 : runs.n);
+  }
+  __syncwarp();
+  return true;
+}
+
 // Everything for seed t with one warp and its workspace slot: the result
 // record (as dibella_xdrop_batch writes it, without the best-of-pair flag) and
 // the run-length encoded columns from (begin_a, begin_b') to (end_a, end_b').
-// Every lane runs both extensions; lane 0 walks back and writes.
+// Every lane runs both extensions; lane 0 walks back and writes.  NB > 0: in the
+// bit-sliced form where its window holds the bands.
+template <int NB>
 __device__ void tb_seed(const TbArgs& p, long long t, char* scratch) {
   const int lane = threadIdx.x & 31;
   const dibella_pair_t pr = p.pairs[t];
@@ -293,6 +730,7 @@ __device__ void tb_seed(const TbArgs& p, long long t, char* scratch) {
     }
     return;
   }
+  if (NB > 0 && tb_seed_bits<(NB > 0 ? NB : 4)>(p, t, scratch, pr, lenA, lenB)) return;
   const long long fA = p.word_offsets[pr.read_a] * 16;
   const long long fB = p.word_offsets[pr.read_b] * 16;
   const long long bp0 = pr.strand ? fB + tb_copy_words(lenB) * 16 : fB;  // B': forward or reverse-complement copy
@@ -355,11 +793,12 @@ __device__ void tb_seed(const TbArgs& p, long long t, char* scratch) {
 
 // A warp per seed: warp w (of n_lanes warps, one workspace slot each) takes
 // seeds w, w + n_lanes, ...
+template <int NB>
 __global__ void __launch_bounds__(kTbThreads) traceback_kernel(TbArgs p) {
   const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   if (warp >= p.n_lanes) return;
   char* scratch = p.workspace + warp * p.lane_bytes;
-  for (long long t = warp; t < p.n_pairs; t += p.n_lanes) tb_seed(p, t, scratch);
+  for (long long t = warp; t < p.n_pairs; t += p.n_lanes) tb_seed<NB>(p, t, scratch);
 }
 
 long long tb_lane_bytes(long long max_len, long long moves_words) {
@@ -422,8 +861,19 @@ int dibella_xdrop_traceback(const uint32_t* packed_words, const int64_t* read_wo
   a.moves_words = moves_words;
   a.workspace = (char*)workspace;
   a.lane_bytes = tb_lane_bytes(max_read_len, moves_words);
+  // The bit-sliced form by the planes that X needs, as the batch does.
+  const bool unit = a.M == 1 && a.S == -1 && a.G == -1 && a.X >= 1 && a.X <= 59;
+  if (unit) {  // four blocks (16 warps) are resident on an SM: more slots would only run after them
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0 &&
+        a.n_lanes > 16ll * sms)
+      a.n_lanes = 16ll * sms;
+  }
   const long long blocks = (a.n_lanes * 32 + kTbThreads - 1) / kTbThreads;
-  traceback_kernel<<<(unsigned)blocks, kTbThreads, 0, (cudaStream_t)stream>>>(a);
+  const auto kernel = !unit ? traceback_kernel<0>
+                            : (a.X <= 11 ? traceback_kernel<4> : (a.X <= 27 ? traceback_kernel<5> : traceback_kernel<6>));
+  kernel<<<(unsigned)blocks, kTbThreads, 0, (cudaStream_t)stream>>>(a);
   return cudaGetLastError() == cudaSuccess ? DIBELLA_OK : DIBELLA_ECUDA;
 }
 

@@ -1594,8 +1594,9 @@ __global__ void __launch_bounds__(NW * 32) narrow_kernel(ExtendParams p) {
 }
 
 #include "xdrop_bits.cuh"
+#include "xdrop_bits_run.cuh"
 
-// Bit-sliced form (see xdrop_bits.cuh).  Four blocks would fit an SM, two or one
+// Bit-sliced form (see xdrop_bits.cuh, xdrop_bits_run.cuh).  Four blocks would fit an SM, two or one
 // are launched; asked for no residency, the compiler spilled to 72 registers.
 template <int NB>
 __global__ void __launch_bounds__(kBlockThreads, 4) bits_shared_kernel(ExtendParams p) {

@@ -1,4 +1,4 @@
-// The bit-sliced X-drop kernel (csrc/xdrop_bits.cuh) run on the CPU: 32 lanes as
+// The bit-sliced X-drop kernel (csrc/xdrop_bits.cuh, csrc/xdrop_bits_run.cuh) run on the CPU: 32 lanes as
 // fibers that meet at every warp intrinsic.  Built and driven by
 // tests/test_bits_emulation.py; no GPU, no CUDA headers.
 #include <ucontext.h>
@@ -175,6 +175,7 @@ unsigned pop_warp(Counters* cnt, int q) {
 }
 
 #include "../paper_2001_10049_gb300/csrc/xdrop_bits.cuh"
+#include "../paper_2001_10049_gb300/csrc/xdrop_bits_run.cuh"
 
 ExtendParams g_p;
 int g_form = 0;

@@ -55,3 +55,41 @@ def test_crowded_warps(X):
     for r in (sub, exp):
         r["status"] &= ~4  # the best-of-pair flag depends on the neighbouring records
     assert_same(sub, exp, "oracle, X=%d" % X)
+
+
+@pytest.mark.parametrize("moves_words,ops_per_seed", [(1 << 18, 4096), (30000, 4096), (2500, 4096), (300, 64), (1 << 18, 7)])
+@pytest.mark.parametrize("X", [5, 25, 59])
+def test_traceback_equals_general_form(X, moves_words, ops_per_seed):
+    """Scores and X doubled give the same alignments, but by the general form:
+    every run, run count and status (moves or runs that do not fit among them)
+    is the same, and the scores are doubled.  The capacities take the two
+    extensions together, one after the other, and beyond what fits."""
+    import torch
+    import paper_2001_10049_gb300 as dib
+    rng = random.Random(X + moves_words)
+    rand = lambda n: "".join(rng.choice("ACGT") for _ in range(n))
+
+    def noisy(s, e):
+        out = []
+        for ch in s:
+            r = rng.random()
+            out.append("" if r < 0.3 * e else (rng.choice("ACGT") if r < 0.5 * e else ch + (rng.choice("ACGT") if r < e else "")))
+        return "".join(out)
+
+    core = rand(2500)
+    reads = [noisy(core, 0.15) for _ in range(6)] + [core, core, rand(1800), rand(2000), rand(4) * 300, "A" * 500, rand(40)]
+    reads += [rc(r) for r in reads[:3]]
+    recs = [(a, b, p, min(p, len(reads[b]) - 31), st) for a in range(len(reads)) for b in range(len(reads))
+            for st in (0, 1) for p in (0, len(reads[a]) // 2, max(0, len(reads[a]) - 31))]
+    recs = [r for r in recs if r[3] >= 0]
+    ascii, offs = reads_to_arrays(reads)
+    al = dib.Aligner(dib.ReadStore.from_ascii(ascii, offs), len(recs), k=31)
+    pairs = make_pairs(recs)
+    res, ops, n_ops = al.traceback(pairs, (1, -1, -1, X), ops_per_seed=ops_per_seed, moves_words=moves_words)
+    res2, ops2, n_ops2 = al.traceback(pairs, (2, -2, -2, 2 * X), ops_per_seed=ops_per_seed, moves_words=moves_words)
+    assert np.array_equal(n_ops, n_ops2) and np.array_equal(ops, ops2)
+    for f in ("begin_a", "end_a", "begin_b", "end_b", "status", "cells"):
+        assert np.array_equal(res[f], res2[f]), f
+    for f in ("score", "score_left", "score_right"):
+        assert np.array_equal(2 * res[f], res2[f]), f
+    torch.cuda.synchronize()
