@@ -34,6 +34,13 @@
 //            greedy seed rule along its run;
 //   compact  a scan of the selection flags writes the 24-byte pair records,
 //            sorted by (read_a, read_b, seed_id).
+// Where the code and the occurrence index share one 64-bit word (k = 17 up to
+// 2^30 bases), the count is instead by sorting into buckets and counting each in
+// shared memory (see "counting in buckets"): 142 M occurrences of the E.
+// coli-sized reads, whole call, 8.9 ms against 17.2 with all code digits sorted
+// and a global walk of the runs (6.1 ms of that, an atomic per 32 occurrences on
+// one counter); the call's largest parts now are the radix scatters (3.9 ms, 109
+// G keys/s) and the bucket kernel (2.6 ms).
 // Nothing here waits on another block; every probe loop is bounded.
 
 #include <cuda_runtime.h>
@@ -66,7 +73,7 @@ struct CandState {
   unsigned long long seeds;       // seed records written
   unsigned int status;            // bit 0 table full, bit 1 pair capacity, bit 2 output
                                   // capacity, bit 3 occurrence capacity, bit 4 sort inconsistency
-  unsigned int pad;
+  unsigned int ticket;            // blocks that have finished their part (digit_hist_scan_kernel)
   unsigned long long pass_count;  // partitioned count: occurrences appended in this pass
   unsigned long long pass_held;   // ... capped at the pass capacity
   unsigned long long max_pass;    // ... the largest pass
@@ -454,6 +461,66 @@ void scan_counts(const unsigned int* counts, unsigned long long* offsets, const 
   scan_apply_kernel<<<kScanBlocks, kScanThreads, 0, st>>>(counts, offsets, n_ptr, mode, fixed_len, part);
 }
 
+// Histograms and scan in one launch, for few tiles (kFewTiles): the block that
+// finishes last scans all counts, thread d the tiles of digit d.  A pass of a
+// small sort is bound by its launches, four with the kernels above, two with
+// this one (the 0.5 Mb read set's whole call: 274 us, 557 before).
+constexpr unsigned long long kFewTiles = 512;
+template <typename K>
+__global__ void __launch_bounds__(1024) digit_hist_scan_kernel(const K* __restrict__ keys, const unsigned long long* n_ptr,
+                                                              int shift, unsigned int* hist, unsigned long long* offsets,
+                                                              unsigned int* ticket) {
+  constexpr int kT = KeyOps<K>::kTile;
+  __shared__ unsigned int h[256];
+  __shared__ unsigned long long wsum[8];
+  __shared__ bool last;
+  const unsigned long long n = *n_ptr;
+  const unsigned long long n_tiles = (n + kT - 1) / kT;
+  for (unsigned long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    if (threadIdx.x < 256) h[threadIdx.x] = 0;
+    __syncthreads();
+    const unsigned long long t0 = tile * kT;
+#pragma unroll
+    for (int j = 0; j < kT / 1024; ++j) {
+      const unsigned long long i = t0 + (unsigned long long)j * 1024 + threadIdx.x;
+      if (i < n) atomicAdd(&h[KeyOps<K>::digit(keys[i], shift)], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < 256) hist[(unsigned long long)threadIdx.x * n_tiles + tile] = h[threadIdx.x];
+    __syncthreads();
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool mine = threadIdx.x < 256;
+  const unsigned int* row = hist + (unsigned long long)(threadIdx.x & 255) * n_tiles;
+  unsigned long long sum = 0;
+#pragma unroll 8
+  for (unsigned long long t = 0; t < n_tiles && mine; ++t) sum += __ldcg(row + t);
+  unsigned long long x = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long y = __shfl_up_sync(kFullMask, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31 && mine) wsum[warp] = x;
+  __syncthreads();
+  if (mine) {
+    unsigned long long at = x - sum;
+    for (int w = 0; w < warp; ++w) at += wsum[w];
+    unsigned long long* out = offsets + (unsigned long long)threadIdx.x * n_tiles;
+#pragma unroll 8
+    for (unsigned long long t = 0; t < n_tiles; ++t) {
+      out[t] = at;
+      at += __ldcg(row + t);
+    }
+  }
+  if (threadIdx.x == 0) *ticket = 0;
+}
+
 // One stable pass of the LSD sort, a tile of kTile keys per block iteration:
 // the tile is copied into shared memory (16-byte asynchronous copies), each
 // warp ranks its contiguous kWarpKeys keys by digit (counts, then a prefix over
@@ -462,12 +529,13 @@ void scan_counts(const unsigned int* counts, unsigned long long* offsets, const 
 // order so that each digit's keys go to consecutive addresses.  A destination
 // outside [0, n) (counts that disagree with the histogram) is skipped and
 // flagged in status bit 4.
+// NT threads: 256, two blocks per SM, or for few tiles 1,024 (a small sort is as
+// long as its tiles take: 15 us a tile with 256).
 constexpr int kScatterThreads = 256;
 constexpr int kScatterBlocksPerSM = 2;
-constexpr int kScatterWarps = kScatterThreads / 32;
-template <typename K>
+template <typename K, int NT = kScatterThreads>
 constexpr size_t scatter_smem() {
-  return (size_t)KeyOps<K>::kTile * sizeof(K) + (size_t)KeyOps<K>::kTile * 2 + (size_t)kScatterWarps * 256 * 4 +
+  return (size_t)KeyOps<K>::kTile * sizeof(K) + (size_t)KeyOps<K>::kTile * 2 + (size_t)(NT / 32) * 256 * 4 +
          256 * 8 + 256 * 4;
 }
 static_assert(KeyOps<unsigned long long>::kTile <= 65536 && KeyOps<Key2>::kTile <= 65536, "tile indices are 16-bit");
@@ -483,11 +551,12 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src,
 
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-template <typename K>
-__global__ void __launch_bounds__(kScatterThreads, kScatterBlocksPerSM)
+template <typename K, int NT = kScatterThreads>
+__global__ void __launch_bounds__(NT, NT == kScatterThreads ? kScatterBlocksPerSM : 1)
     digit_scatter_kernel(const K* __restrict__ in, K* __restrict__ out, const unsigned long long* n_ptr, int shift,
                          const unsigned long long* offsets, unsigned int* status) {
   constexpr int kT = KeyOps<K>::kTile;
+  constexpr int kScatterWarps = NT / 32;
   constexpr int kWarpKeys = kT / kScatterWarps;
   constexpr int kPerChunk = 16 / (int)sizeof(K);  // keys per 16-byte copy
   extern __shared__ __align__(16) unsigned char smem[];
@@ -504,13 +573,13 @@ __global__ void __launch_bounds__(kScatterThreads, kScatterBlocksPerSM)
   for (unsigned long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const unsigned long long t0 = tile * kT;
     const int m = n - t0 < (unsigned long long)kT ? (int)(n - t0) : kT;
-    for (int c = threadIdx.x; c < kT / kPerChunk; c += kScatterThreads) {
+    for (int c = threadIdx.x; c < kT / kPerChunk; c += NT) {
       const int e = kPerChunk * c;  // a 16-byte chunk: keys e .. e + kPerChunk - 1, zero-filled past the tile's end
       const int valid = m - e < kPerChunk ? (m - e > 0 ? m - e : 0) : kPerChunk;
       const unsigned bytes = (unsigned)valid * (unsigned)sizeof(K);
       cp_async16(skey + e, bytes ? (const void*)(in + t0 + e) : (const void*)in, bytes);
     }
-    for (int x = threadIdx.x; x < kScatterWarps * 256; x += kScatterThreads) wcnt[x] = 0;
+    for (int x = threadIdx.x; x < kScatterWarps * 256; x += NT) wcnt[x] = 0;
     cp_async_wait_all();
     __syncthreads();
     for (int r = 0; r < kWarpKeys; r += 32) {
@@ -547,7 +616,7 @@ __global__ void __launch_bounds__(kScatterThreads, kScatterBlocksPerSM)
       }
     }
     __syncthreads();
-    for (int x = threadIdx.x; x < kScatterWarps * 256; x += kScatterThreads) wcnt[x] += lstart[x & 255];
+    for (int x = threadIdx.x; x < kScatterWarps * 256; x += NT) wcnt[x] += lstart[x & 255];
     __syncthreads();
     unsigned int* next = wcnt + warp * 256;  // this warp's next slot per digit
     for (int r = 0; r < kWarpKeys; r += 32) {
@@ -563,7 +632,7 @@ __global__ void __launch_bounds__(kScatterThreads, kScatterBlocksPerSM)
       if (ok && c + rank < (unsigned)kT) inv[c + rank] = (unsigned short)i;
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < m; q += kScatterThreads) {
+    for (int q = threadIdx.x; q < m; q += NT) {
       const K key = skey[inv[q] & (kT - 1)];
       const unsigned d = KeyOps<K>::digit(key, shift);
       const unsigned long long g = gbase[d] + (unsigned long long)(q - (int)lstart[d]);
@@ -576,25 +645,37 @@ __global__ void __launch_bounds__(kScatterThreads, kScatterBlocksPerSM)
   }
 }
 
+template <typename K, int NT>
+cudaError_t set_scatter_smem_of() {
+  return cudaFuncSetAttribute(digit_scatter_kernel<K, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)scatter_smem<K, NT>());
+}
 cudaError_t set_scatter_smem() {
-  cudaError_t e = cudaFuncSetAttribute(digit_scatter_kernel<unsigned long long>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)scatter_smem<unsigned long long>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(digit_scatter_kernel<Key2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)scatter_smem<Key2>());
-  return e;
+  cudaError_t e;
+  if ((e = set_scatter_smem_of<unsigned long long, kScatterThreads>()) != cudaSuccess ||
+      (e = set_scatter_smem_of<Key2, kScatterThreads>()) != cudaSuccess ||
+      (e = set_scatter_smem_of<unsigned long long, 1024>()) != cudaSuccess)
+    return e;
+  return set_scatter_smem_of<Key2, 1024>();
 }
 
 // One stable LSD pass by the digit at `shift`: histogram, scan, scatter.
+// `tiles_max` bounds the sort tiles that the keys can take.
 template <typename K>
 void radix_pass(const K* src, K* dst, const unsigned long long* n_ptr, int shift, unsigned int* hist,
-                unsigned long long* hoff, unsigned long long tiles_max, unsigned long long* part,
-                unsigned int* status, int sms, cudaStream_t st) {
+                unsigned long long* hoff, unsigned long long tiles_max, unsigned long long* part, CandState* state,
+                int sms, cudaStream_t st) {
+  if (tiles_max <= kFewTiles) {
+    const unsigned hb = (unsigned)(tiles_max < (unsigned long long)sms ? (tiles_max > 0 ? tiles_max : 1) : sms);
+    digit_hist_scan_kernel<K><<<hb, 1024, 0, st>>>(src, n_ptr, shift, hist, hoff, &state->ticket);
+    digit_scatter_kernel<K, 1024><<<hb, 1024, scatter_smem<K, 1024>(), st>>>(src, dst, n_ptr, shift, hoff,
+                                                                            &state->status);
+    return;
+  }
   digit_hist_kernel<K><<<sms * 8, 256, 0, st>>>(src, n_ptr, shift, hist, tiles_max);
   scan_counts(hist, hoff, n_ptr, 1, (unsigned long long)KeyOps<K>::kTile, part, st);
   digit_scatter_kernel<K><<<sms * kScatterBlocksPerSM, kScatterThreads, scatter_smem<K>(), st>>>(
-      src, dst, n_ptr, shift, hoff, status);
+      src, dst, n_ptr, shift, hoff, &state->status);
 }
 
 // ---- sort-based count (when code and occurrence index share 64 bits) ----------
@@ -619,8 +700,18 @@ __global__ void occ_total_kernel(const unsigned int* cnt, const unsigned long lo
   st->instances = total;
 }
 
-// Every occurrence as (canonical code << ib | occurrence index), and its read,
-// position and orientation under that index.
+// A bijection of the 2k-bit codes that spreads them evenly over the buckets (the
+// highest bits of the result): equal codes stay equal, and nothing else of the
+// code is used after this.
+__device__ __forceinline__ unsigned long long mix_code(unsigned long long c, unsigned long long code_mask) {
+  return (c * 0x9E3779B97F4A7C15ull) & code_mask;
+}
+__host__ __device__ inline unsigned long long code_mask_of(int k) {
+  return k == 32 ? ~0ull : (1ull << (2 * k)) - 1ull;
+}
+
+// Every occurrence as (mixed canonical code << ib | occurrence index), and its read,
+// position and orientation under that index.  gridDim.y warps share a read.
 __global__ void extract_kernel(StoreRef sr, const unsigned long long* off, int ib, unsigned long long cap,
                                unsigned long long* keys, unsigned long long* info) {
   const int lane = threadIdx.x & 31;
@@ -630,79 +721,306 @@ __global__ void extract_kernel(StoreRef sr, const unsigned long long* off, int i
     const long long len = sr.lengths[r];
     const long long first = sr.word_offsets[r] * 16;
     const unsigned long long o = off[r];
-    for (long long p = lane; p + sr.k <= len; p += 32) {
+    for (long long p = 32 * blockIdx.y + lane; p + sr.k <= len; p += 32 * gridDim.y) {
       unsigned orient;
       const unsigned long long c = canonical(bases_le(sr.words, first + p, sr.k), sr.k, &orient);
       const unsigned long long idx = o + (unsigned long long)p;
       if (idx >= cap) break;  // n_bases understated (status bit 3)
-      keys[idx] = (c << ib) | idx;
+      keys[idx] = (mix_code(c, code_mask_of(sr.k)) << ib) | idx;
       info[idx] = ((unsigned long long)r << 32) | ((unsigned long long)p << 1) | orient;
     }
   }
 }
 
-// A thread per run of equal codes in the sorted occurrences (n_ptr of them):
-// the multiplicity, and for a retained k-mer its occurrence pairs (as in
-// emit_pairs_kernel), as one-word or two-word keys.
-template <typename K>
-__global__ void run_emit_kernel(const unsigned long long* __restrict__ sorted, const unsigned long long* info, int ib,
-                                int mult_lo, int mult_hi, KeyLayout kl, K* keys_out,
-                                unsigned long long capacity, const unsigned long long* n_ptr, CandState* st) {
+// ---- counting in buckets -----------------------------------------------------
+// The occurrences are sorted only by the highest bucket_bits of their mixed
+// code; a bucket of about kBucketMean occurrences is then counted in a block's
+// shared memory.  Sorting all 34 bits of a 17-mer takes 5 passes over the keys
+// (24 bytes each per key), this takes 2 and one read of each bucket, from which
+// the pairs are emitted too, with one global atomic per bucket and counter.
+constexpr int kBucketMean = 2048;
+constexpr int kBucketThreads = 256;
+constexpr int kBucketSlots = 4096;  // hash table slots: twice the occurrences of a mean bucket
+constexpr int kBucketSeg = 2048;    // retained occurrences held in shared memory (else in the spare key buffer)
+constexpr int kBucketProbes = 96;
+constexpr int kBucketBlocksPerSM = 3;
+constexpr int kBucketHeld = 12;     // occurrences that a thread holds in registers (buckets up to 3,072)
+
+// Bits of the mixed code that number the buckets of up to n occurrences.
+int bucket_bits(unsigned long long n, int k) {
+  int b = 0;
+  while (b < 16 && b < 2 * k && (n >> b) > (unsigned long long)kBucketMean) ++b;
+  return b;
+}
+
+// starts[b] = the first occurrence of bucket b, for b = 0 .. n_buckets (the
+// occurrences are in bucket order; `shift` brings a key's bucket to bit 0).
+__global__ void bucket_starts_kernel(const unsigned long long* __restrict__ keys, const unsigned long long* n_ptr,
+                                     int shift, unsigned n_buckets, unsigned long long* starts) {
   const unsigned long long n = *n_ptr;
-  const unsigned long long imask = (1ull << ib) - 1ull;
-  const unsigned long long lane = threadIdx.x & 31;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-  for (unsigned long long w0 = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) - lane; w0 < n;
-       w0 += stride) {
-    const unsigned long long i = w0 + lane;
-    bool keep = false;
-    int c = 0;
-    if (i < n && (i == 0 || (sorted[i - 1] >> ib) != (sorted[i] >> ib))) {
-      const unsigned long long code = sorted[i] >> ib;
-      unsigned long long e = i + 1;
-      while (e < n && (sorted[e] >> ib) == code && e - i <= (unsigned long long)mult_hi) ++e;
-      const unsigned long long mult = e - i;  // capped at mult_hi + 1: enough to reject
-      keep = mult >= (unsigned long long)mult_lo && mult <= (unsigned long long)mult_hi;
-      c = keep ? (int)mult : 0;
-    }
-    warp_atomic_add(&st->retained, keep ? 1u : 0u);
-    unsigned long long v[kMaxMult];
-    int n_pairs = 0;
-    if (keep) {
-      for (int x = 0; x < c; ++x) v[x] = info[sorted[i + x] & imask];
-      for (int x = 1; x < c; ++x) {
-        const unsigned long long t = v[x];
-        int y = x - 1;
-        while (y >= 0 && v[y] > t) {
-          v[y + 1] = v[y];
-          --y;
-        }
-        v[y + 1] = t;
-      }
-      for (int x = 0; x < c; ++x)
-        for (int y = x + 1; y < c; ++y) n_pairs += (v[x] >> 32) != (v[y] >> 32);
-    }
-    const unsigned long long at = warp_atomic_add(&st->occ_pairs, (unsigned long long)n_pairs);
-    if (n_pairs == 0) continue;
-    if (at + n_pairs > capacity) {
-      atomicOr(&st->status, 2u);
-      continue;
-    }
-    unsigned long long o = at;
-    for (int x = 0; x < c; ++x)
-      for (int y = x + 1; y < c; ++y) {
-        const unsigned long long ra = v[x] >> 32, rb = v[y] >> 32;
-        if (ra == rb) continue;
-        const unsigned long long pa = (v[x] >> 1) & 0x7FFFFFFFull, pb = (v[y] >> 1) & 0x7FFFFFFFull;
-        const unsigned long long strand = (v[x] ^ v[y]) & 1ull;
-        keys_out[o++] = make_key(kl, ra, rb, pa, pb, strand, (K*)nullptr);
-      }
+  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i <= n; i += stride) {
+    const unsigned lo = i == 0 ? 0u : (shift < 64 ? (unsigned)(keys[i - 1] >> shift) : 0u) + 1u;
+    const unsigned hi = i == n ? n_buckets : (shift < 64 ? (unsigned)(keys[i] >> shift) : 0u);
+    for (unsigned b = lo; b <= hi; ++b) starts[b] = i;
   }
+}
+
+// Exclusive sum of v over the block (kBucketThreads threads); *total gets the whole.
+__device__ __forceinline__ unsigned bucket_scan(unsigned v, unsigned* wsum, unsigned* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned x = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(kFullMask, x, o);
+    if (lane >= o) x += y;
+  }
+  __syncthreads();
+  if (lane == 31) wsum[warp] = x;
+  __syncthreads();
+  unsigned before = 0, all = 0;
+  for (int w = 0; w < kBucketThreads / 32; ++w) {
+    before += w < warp ? wsum[w] : 0u;
+    all += wsum[w];
+  }
+  *total = all;
+  return before + x - v;
+}
+
+// A block per bucket: count its codes, then form the occurrence pairs of the
+// retained ones (as emit_pairs_kernel does), as one-word or two-word keys.  A
+// bucket with more distinct codes than the table takes is counted in parts, by
+// the next bits of the code, halved until each part fits.  Tag: 32 bits where
+// the rest of the code fits.
+template <typename K, typename Tag>
+__global__ void __launch_bounds__(kBucketThreads, kBucketBlocksPerSM) bucket_emit_kernel(
+    const unsigned long long* __restrict__ keys, const unsigned long long* __restrict__ info, unsigned long long* spare,
+    const unsigned long long* starts, unsigned n_buckets, int ib, int rest_bits, int mult_lo, int mult_hi, KeyLayout kl,
+    K* keys_out, unsigned long long capacity, CandState* st) {
+  extern __shared__ __align__(16) unsigned char bsm[];
+  unsigned long long* seg_s = (unsigned long long*)bsm;
+  Tag* tag = (Tag*)(seg_s + kBucketSeg);
+  // per slot: the count; then, for a retained code, first place << 12 | count << 6 | places taken, else 0
+  unsigned* slot = (unsigned*)(tag + kBucketSlots);
+  unsigned* list = slot + kBucketSlots;  // the retained codes: first place << 6 | count
+  __shared__ unsigned wsum[kBucketThreads / 32];
+  __shared__ int overflow;
+  __shared__ unsigned long long out_at;
+  constexpr int kPer = kBucketSlots / kBucketThreads;
+  const unsigned long long imask = (1ull << ib) - 1ull;
+  const unsigned long long rmask = rest_bits == 64 ? ~0ull : (1ull << rest_bits) - 1ull;
+  unsigned long long kept_codes = 0;
+  for (unsigned b = blockIdx.x; b < n_buckets; b += gridDim.x) {
+    const unsigned long long lo = starts[b], hi = starts[b + 1];
+    if (lo == hi) continue;  // (uniform)
+    int j = 0;
+    for (unsigned long long part = 0;;) {
+      // ---- count the codes whose highest j bits of the rest are `part` ----
+      for (int s = threadIdx.x; s < kBucketSlots; s += kBucketThreads) {
+        tag[s] = 0;
+        slot[s] = 0;
+      }
+      if (threadIdx.x == 0) overflow = 0;
+      __syncthreads();
+      auto find = [&](unsigned long long rest, bool insert) -> int {
+        const Tag t = (Tag)(rest + 1);
+        unsigned s = (unsigned)((rest * 0xD6E8FEB86659FD93ull) >> 40) & (kBucketSlots - 1);
+        for (int q = 0; q < kBucketProbes; ++q) {
+          Tag c = tag[s];
+          if (c == 0 && insert) c = atomicCAS(&tag[s], (Tag)0, t);
+          if (c == t || c == 0) return (int)s;  // (c == 0: just inserted)
+          s = (s + 1) & (kBucketSlots - 1);
+        }
+        return -1;
+      };
+      const bool held = j == 0 && hi - lo <= (unsigned long long)(kBucketHeld * kBucketThreads);
+      unsigned long long mine[kBucketHeld];  // held: this thread's keys, then (in the low bits) their slots
+      auto count = [&](unsigned long long rest) -> int {
+        const int s = find(rest, true);
+        if (s < 0)
+          overflow = 1;
+        else if (slot[s] <= (unsigned)mult_hi)  // (one too many is enough: no pile-up on a frequent code)
+          atomicAdd(&slot[s], 1u);
+        return s;
+      };
+      if (held) {
+#pragma unroll
+        for (int q = 0; q < kBucketHeld; ++q) {
+          const unsigned long long i = lo + q * kBucketThreads + threadIdx.x;
+          mine[q] = i < hi ? keys[i] : ~0ull;
+        }
+#pragma unroll
+        for (int q = 0; q < kBucketHeld; ++q) {
+          if (lo + q * kBucketThreads + threadIdx.x < hi) {
+            const int s = count((mine[q] >> ib) & rmask);
+            mine[q] = ((mine[q] & imask) << 12) | (unsigned)(s & (kBucketSlots - 1));
+          }
+        }
+      } else {
+#pragma unroll 4
+        for (unsigned long long i = lo + threadIdx.x; i < hi; i += kBucketThreads) {
+          const unsigned long long rest = (keys[i] >> ib) & rmask;
+          if (j > 0 && (rest >> (rest_bits - j)) != part) continue;
+          count(rest);
+        }
+      }
+      __syncthreads();
+      if (overflow && j < rest_bits) {  // (uniform; at j = rest_bits a part is one code)
+        ++j;
+        part <<= 1;
+        __syncthreads();
+        continue;
+      }
+      // ---- places of the retained codes' occurrences ----
+      unsigned occ = 0, codes = 0;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const unsigned c = slot[q * kBucketThreads + threadIdx.x];
+        if (c >= (unsigned)mult_lo && c <= (unsigned)mult_hi) {
+          occ += c;
+          ++codes;
+        }
+      }
+      unsigned both;  // occurrences (18 bits) and codes of the part
+      unsigned at = bucket_scan(occ | (codes << 18), wsum, &both);
+      const unsigned total = both & 0x3FFFFu, n_codes = both >> 18;
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const unsigned c = slot[q * kBucketThreads + threadIdx.x];
+        const bool keep = c >= (unsigned)mult_lo && c <= (unsigned)mult_hi;
+        slot[q * kBucketThreads + threadIdx.x] = keep ? ((at & 0x3FFFFu) << 12) | (c << 6) : 0u;
+        if (keep) {
+          list[at >> 18] = ((at & 0x3FFFFu) << 6) | c;
+          at += c | (1u << 18);
+        }
+      }
+      kept_codes += codes;
+      unsigned long long* seg = total <= (unsigned)kBucketSeg ? seg_s : spare + lo;
+      __syncthreads();
+      if (total > 0) {  // (uniform)
+        if (held) {
+          unsigned long long word[kBucketHeld];
+#pragma unroll
+          for (int q = 0; q < kBucketHeld; ++q) {
+            const bool keep = lo + q * kBucketThreads + threadIdx.x < hi && slot[mine[q] & (kBucketSlots - 1)] != 0;
+            mine[q] = keep ? mine[q] : ~0ull;
+            word[q] = keep ? info[mine[q] >> 12] : 0ull;
+          }
+#pragma unroll
+          for (int q = 0; q < kBucketHeld; ++q) {
+            if (mine[q] != ~0ull) {
+              const unsigned v = atomicAdd(&slot[mine[q] & (kBucketSlots - 1)], 1u);
+              seg[(v >> 12) + (v & 63u)] = word[q];
+            }
+          }
+        } else {
+          for (unsigned long long i = lo + threadIdx.x; i < hi; i += kBucketThreads) {
+            const unsigned long long key = keys[i], rest = (key >> ib) & rmask;
+            if (j > 0 && (rest >> (rest_bits - j)) != part) continue;
+            const int s = find(rest, false);
+            if (s < 0 || slot[s] == 0) continue;
+            const unsigned v = atomicAdd(&slot[s], 1u);
+            seg[(v >> 12) + (v & 63u)] = info[key & imask];
+          }
+        }
+        __syncthreads();
+        // ---- order each code's occurrences, and its pairs ----
+        unsigned n_pairs = 0;
+        for (unsigned q = threadIdx.x; q < n_codes; q += kBucketThreads) {
+          const int c = (int)(list[q] & 63u);
+          unsigned long long* o = seg + (list[q] >> 6);
+          for (int x = 1; x < c; ++x) {
+            const unsigned long long e = o[x];
+            int y = x - 1;
+            for (; y >= 0 && o[y] > e; --y) o[y + 1] = o[y];
+            o[y + 1] = e;
+          }
+          for (int x = 0; x < c; ++x)
+            for (int y = x + 1; y < c; ++y) n_pairs += (o[x] >> 32) != (o[y] >> 32);
+        }
+        unsigned all;
+        const unsigned mine = bucket_scan(n_pairs, wsum, &all);
+        if (threadIdx.x == 0 && all > 0) out_at = atomicAdd(&st->occ_pairs, (unsigned long long)all);
+        __syncthreads();
+        unsigned long long w = out_at + mine;
+        if (n_pairs > 0 && w + n_pairs > capacity) {
+          atomicOr(&st->status, 2u);
+          n_pairs = 0;
+        }
+        for (unsigned q = threadIdx.x; q < n_codes && n_pairs > 0; q += kBucketThreads) {
+          const int c = (int)(list[q] & 63u);
+          const unsigned long long* o = seg + (list[q] >> 6);
+          for (int x = 0; x < c; ++x)
+            for (int y = x + 1; y < c; ++y) {
+              const unsigned long long e = o[x], f = o[y], ra = e >> 32, rb = f >> 32;
+              if (ra == rb) continue;
+              keys_out[w++] = make_key(kl, ra, rb, (e >> 1) & 0x7FFFFFFFull, (f >> 1) & 0x7FFFFFFFull, (e ^ f) & 1ull,
+                                       (K*)nullptr);
+            }
+        }
+      }
+      __syncthreads();
+      // ---- the next part ----
+      ++part;
+      while (j > 0 && (part & 1ull) == 0) {
+        --j;
+        part >>= 1;
+      }
+      if (j == 0) break;
+    }
+  }
+  kept_codes = warp_atomic_add(&st->retained, kept_codes);
+}
+
+template <typename Tag>
+constexpr size_t bucket_smem() {
+  return (size_t)kBucketSeg * 8 + (size_t)kBucketSlots * (sizeof(Tag) + 8);
+}
+
+// Orders n_ptr occurrences (at most n_max; in buf0, buf1 spare) by bucket and emits
+// their pairs.  Keys: mixed code << ib | index.
+template <typename K>
+cudaError_t count_in_buckets(unsigned long long* buf0, unsigned long long* buf1, const unsigned long long* info,
+                             const unsigned long long* n_ptr, unsigned long long n_max, int k, int ib, int mult_lo,
+                             int mult_hi, const KeyLayout& kl, K* keys_out, unsigned long long capacity,
+                             unsigned int* hist, unsigned long long* hoff, unsigned long long* part, CandState* state,
+                             int sms, cudaStream_t st) {
+  const int bits = bucket_bits(n_max, k), rest_bits = 2 * k - bits;
+  const unsigned long long tiles = (n_max + KeyOps<unsigned long long>::kTile - 1) / KeyOps<unsigned long long>::kTile;
+  for (int j = 0; j < (bits + 7) / 8; ++j) {
+    radix_pass(buf0, buf1, n_ptr, ib + rest_bits + 8 * j, hist, hoff, tiles, part, state, sms, st);
+    unsigned long long* tmp = buf0;
+    buf0 = buf1;
+    buf1 = tmp;
+  }
+  const unsigned n_buckets = 1u << bits;
+  unsigned long long* starts = hoff;  // the last pass has read its offsets; n_buckets + 1 <= 256 tiles entries
+  bucket_starts_kernel<<<sms * 8, 256, 0, st>>>(buf0, n_ptr, ib + rest_bits, n_buckets, starts);
+  // 64 KB of shared memory a block, 80 with 64-bit tags
+  const unsigned resident = (unsigned)(sms * (rest_bits < 32 ? kBucketBlocksPerSM : 2));
+  const unsigned blocks = n_buckets < resident ? n_buckets : resident;
+  cudaError_t e;
+  if (rest_bits < 32) {
+    const auto fn = bucket_emit_kernel<K, unsigned int>;
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bucket_smem<unsigned int>())) !=
+        cudaSuccess)
+      return e;
+    fn<<<blocks, kBucketThreads, bucket_smem<unsigned int>(), st>>>(buf0, info, buf1, starts, n_buckets, ib, rest_bits,
+                                                                    mult_lo, mult_hi, kl, keys_out, capacity, state);
+  } else {
+    const auto fn = bucket_emit_kernel<K, unsigned long long>;
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)bucket_smem<unsigned long long>())) != cudaSuccess)
+      return e;
+    fn<<<blocks, kBucketThreads, bucket_smem<unsigned long long>(), st>>>(
+        buf0, info, buf1, starts, n_buckets, ib, rest_bits, mult_lo, mult_hi, kl, keys_out, capacity, state);
+  }
+  return cudaGetLastError();
 }
 
 // The partitioned count: one pass per hash part of the canonical codes.  Every
 // occurrence whose code falls in part `part` of n_parts is appended (one
-// warp-aggregated atomic per 32 positions) as (code << ib | slot) with its
+// warp-aggregated atomic per 512 positions: with one per 32 this kernel waited on
+// that counter, 4.9 ms a pass over 206 Mb) as (code << ib | slot) with its
 // read, position and orientation under that slot; the order within a pass is
 // free, since each run is ordered by (read, position) before its pairs are
 // formed and the pairs are sorted afterwards.
@@ -710,6 +1028,7 @@ __device__ __forceinline__ unsigned part_of(unsigned long long code, unsigned n_
   return (unsigned)__umul64hi(mix64(code + 0x9E3779B97F4A7C15ull), (unsigned long long)n_parts);
 }
 
+constexpr int kPartSteps = 16;
 __global__ void extract_part_kernel(StoreRef sr, unsigned part, unsigned n_parts, int ib, unsigned long long cap,
                                     unsigned long long* keys, unsigned long long* info, CandState* st) {
   const int lane = threadIdx.x & 31;
@@ -719,28 +1038,38 @@ __global__ void extract_part_kernel(StoreRef sr, unsigned part, unsigned n_parts
   for (long long r = warp; r < sr.n_reads; r += n_warps) {
     const long long len = sr.lengths[r];
     const long long first = sr.word_offsets[r] * 16;
-    for (long long p0 = 0; p0 + sr.k <= len; p0 += 32) {  // uniform over the warp
-      const long long p = p0 + lane;
-      unsigned orient = 0;
-      unsigned long long c = 0;
-      bool mine = false;
-      if (p + sr.k <= len) {
-        c = canonical(bases_le(sr.words, first + p, sr.k), sr.k, &orient);
-        mine = part_of(c, n_parts) == part;
+    for (long long p0 = 0; p0 + sr.k <= len; p0 += 32 * kPartSteps) {  // uniform over the warp
+      unsigned long long c[kPartSteps];
+      unsigned mine = 0, orients = 0, total = 0, before[kPartSteps];
+#pragma unroll
+      for (int q = 0; q < kPartSteps; ++q) {
+        const long long p = p0 + 32 * q + lane;
+        c[q] = 0;
+        if (p + sr.k <= len) {
+          unsigned orient;
+          c[q] = canonical(bases_le(sr.words, first + p, sr.k), sr.k, &orient);
+          orients |= orient << q;
+          mine |= (part_of(c[q], n_parts) == part ? 1u : 0u) << q;
+        }
+        const unsigned bal = __ballot_sync(kFullMask, (mine >> q) & 1u);
+        before[q] = total + __popc(bal & lt);
+        total += __popc(bal);
       }
-      const unsigned bal = __ballot_sync(kFullMask, mine);
-      if (!bal) continue;
+      if (total == 0) continue;
       unsigned long long base = 0;
-      if (lane == 0) base = atomicAdd(&st->pass_count, (unsigned long long)__popc(bal));
+      if (lane == 0) base = atomicAdd(&st->pass_count, (unsigned long long)total);
       base = __shfl_sync(kFullMask, base, 0);
-      if (!mine) continue;
-      const unsigned long long idx = base + __popc(bal & lt);
-      if (idx >= cap) {
-        atomicOr(&st->status, 8u);
-        continue;
+#pragma unroll
+      for (int q = 0; q < kPartSteps; ++q) {
+        if (!((mine >> q) & 1u)) continue;
+        const unsigned long long idx = base + before[q];
+        if (idx >= cap) {
+          atomicOr(&st->status, 8u);
+          continue;
+        }
+        keys[idx] = (mix_code(c[q], code_mask_of(sr.k)) << ib) | idx;
+        info[idx] = ((unsigned long long)r << 32) | ((unsigned long long)(p0 + 32 * q + lane) << 1) | ((orients >> q) & 1u);
       }
-      keys[idx] = (c << ib) | idx;
-      info[idx] = ((unsigned long long)r << 32) | ((unsigned long long)p << 1) | orient;
     }
   }
 }
@@ -757,33 +1086,43 @@ __global__ void pass_end_kernel(CandState* st, unsigned long long cap) {
 
 // ---- seed selection and compaction -----------------------------------------
 
-// A thread per run start walks its run: selection flags and seed ids.
+// Every key's selection flag starts at 0.
+__global__ void clear_flags_kernel(const CandState* st, unsigned int* flags) {
+  const unsigned long long n = st->n_keys;
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n; i += stride)
+    flags[i] = 0u;
+}
+
+// A thread per run start walks its run up to its last seed: selection flags
+// and seed ids of the keys taken.
 template <typename K>
 __global__ void select_kernel(const K* __restrict__ keys, CandState* st, KeyLayout kl,
                               int max_seeds, int gap, unsigned int* flags, unsigned int* sid) {
   const unsigned long long n = st->n_keys;
   const unsigned long long lane = threadIdx.x & 31;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  unsigned long long starts = 0;  // added up at the end: an atomic per 32 keys was most of this kernel's time
   for (unsigned long long w0 = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) - lane; w0 < n;
        w0 += stride) {
     const unsigned long long i = w0 + lane;
     const bool start = i < n && (i == 0 || run_of(kl, keys[i - 1]) != run_of(kl, keys[i]));
-    warp_atomic_add(&st->candidates, start ? 1u : 0u);
     if (!start) continue;
+    ++starts;
     const unsigned long long run = run_of(kl, keys[i]);
     int taken = 0;
     long long last = 0;
-    for (unsigned long long u = i; u < n && run_of(kl, keys[u]) == run; ++u) {
+    for (unsigned long long u = i; u < n && taken < max_seeds && run_of(kl, keys[u]) == run; ++u) {
       const long long pa = (long long)((lo_word(keys[u]) >> kl.sh_pa) & kl.m_pos);
-      const bool take = taken < max_seeds && (taken == 0 || pa >= last + gap);
-      flags[u] = take ? 1u : 0u;
-      sid[u] = take ? (unsigned)taken : 0u;
-      if (take) {
+      if (taken == 0 || pa >= last + gap) {
+        flags[u] = 1u;
+        sid[u] = (unsigned)taken;
         last = pa;
         ++taken;
       }
     }
   }
+  warp_atomic_add(&st->candidates, starts);
 }
 
 // Per-tile sums of the flags.
@@ -812,7 +1151,8 @@ template <typename K>
 __global__ void compact_kernel(const K* __restrict__ keys, const unsigned int* flags,
                                const unsigned int* sid, const unsigned long long* tile_off, CandState* st,
                                KeyLayout kl, dibella_pair_t* out, unsigned long long capacity) {
-  __shared__ unsigned int s[kSortThreads];
+  static_assert(kSortThreads == kBucketThreads, "bucket_scan works on blocks of kBucketThreads");
+  __shared__ unsigned int s[kSortThreads / 32];
   const unsigned long long n = st->n_keys;
   const unsigned long long n_tiles = (n + kTile - 1) / kTile;
   for (unsigned long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
@@ -820,18 +1160,8 @@ __global__ void compact_kernel(const K* __restrict__ keys, const unsigned int* f
     unsigned int v = 0;
     for (int j = 0; j < kSortItems; ++j)
       if (i0 + j < n) v += flags[i0 + j];
-    s[threadIdx.x] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {  // exclusive scan of the 256 thread sums
-      unsigned int acc = 0;
-      for (int t = 0; t < kSortThreads; ++t) {
-        const unsigned int x = s[t];
-        s[t] = acc;
-        acc += x;
-      }
-    }
-    __syncthreads();
-    unsigned long long o = tile_off[tile] + s[threadIdx.x];
+    unsigned int all;
+    unsigned long long o = tile_off[tile] + bucket_scan(v, s, &all);
     for (int j = 0; j < kSortItems; ++j) {
       const unsigned long long i = i0 + j;
       if (i >= n || !flags[i]) continue;
@@ -910,7 +1240,8 @@ CandLayout cand_layout(long long n_reads, long long n_bases, int k, int mult_hi)
   L.slots = slots;
   L.inst = inst;
   L.pairs = inst * (unsigned long long)(mult_hi > 1 ? mult_hi - 1 : 1) / 2 + 1;
-  const unsigned long long ptiles = (L.pairs + kTile - 1) / kTile, otiles = (inst + kTile - 1) / kTile;
+  constexpr unsigned long long kT = KeyOps<unsigned long long>::kTile;
+  const unsigned long long ptiles = (L.pairs + kT - 1) / kT, otiles = (inst + kT - 1) / kT;
   L.tiles = ptiles > otiles ? ptiles : otiles;
   size_t off = 0;
   L.state = off;    off = align256(off + sizeof(CandState));
@@ -958,7 +1289,8 @@ PartLayout part_layout(long long n_bases, int n_parts, long long occ_pair_capaci
   L.wide = wide;
   const size_t ksz = wide ? sizeof(Key2) : 8;
   const unsigned long long ktile = wide ? KeyOps<Key2>::kTile : KeyOps<unsigned long long>::kTile;
-  const unsigned long long otiles = (L.pass_cap + kTile - 1) / kTile, ptiles = (L.pairs + ktile - 1) / ktile;
+  constexpr unsigned long long kT = KeyOps<unsigned long long>::kTile;
+  const unsigned long long otiles = (L.pass_cap + kT - 1) / kT, ptiles = (L.pairs + ktile - 1) / ktile;
   L.tiles = otiles > ptiles ? otiles : ptiles;
   const unsigned long long ctiles = (L.pairs + kTile - 1) / kTile;  // compaction tiles
   size_t off = 0;
@@ -994,6 +1326,7 @@ void select_and_compact(const K* keys, CandState* state, const KeyLayout& kl, in
                         unsigned long long* part, dibella_pair_t* pairs_out, long long pairs_capacity,
                         int64_t* counts_out, int sms, cudaStream_t st) {
   const int sort_blocks = sms * 8;
+  clear_flags_kernel<<<sms * 8, 256, 0, st>>>(state, flags);
   select_kernel<K><<<sms * 8, 256, 0, st>>>(keys, state, kl, max_seeds, gap, flags, sid);
   tile_sum_kernel<<<sort_blocks, kSortThreads, 0, st>>>(flags, state, tsum);
   scan_counts(tsum, toff, &state->n_keys, 2, 0, part, st);
@@ -1077,21 +1410,13 @@ int dibella_candidate_pairs_parts(const uint32_t* packed_words, const int64_t* r
     extract_part_kernel<<<sms * 16, 256, 0, st>>>(sr, (unsigned)p, (unsigned)n_parts, ib, L.pass_cap, ok0, info,
                                                   state);
     pass_end_kernel<<<1, 1, 0, st>>>(state, L.pass_cap);
-    unsigned long long* osrc = ok0;
-    unsigned long long* odst = ok1;
-    for (int j = 0; j < (2 * k + 7) / 8; ++j) {
-      radix_pass(osrc, odst, &state->pass_held, ib + 8 * j, hist, hoff, L.tiles, part, &state->status, sms, st);
-      unsigned long long* tmp = osrc;
-      osrc = odst;
-      odst = tmp;
-    }
     if (wide)
-      run_emit_kernel<Key2><<<sms * 8, 256, 0, st>>>(osrc, info, ib, mult_lo, mult_hi, kl, (Key2*)(ws + L.pk0),
-                                                     L.pairs, &state->pass_held, state);
+      e = count_in_buckets(ok0, ok1, info, &state->pass_held, L.pass_cap, k, ib, mult_lo, mult_hi, kl,
+                           (Key2*)(ws + L.pk0), L.pairs, hist, hoff, part, state, sms, st);
     else
-      run_emit_kernel<unsigned long long><<<sms * 8, 256, 0, st>>>(osrc, info, ib, mult_lo, mult_hi, kl,
-                                                                   (unsigned long long*)(ws + L.pk0), L.pairs,
-                                                                   &state->pass_held, state);
+      e = count_in_buckets(ok0, ok1, info, &state->pass_held, L.pass_cap, k, ib, mult_lo, mult_hi, kl,
+                           (unsigned long long*)(ws + L.pk0), L.pairs, hist, hoff, part, state, sms, st);
+    if (e != cudaSuccess) return DIBELLA_ECUDA;
   }
   cap_keys_kernel<<<1, 1, 0, st>>>(state, L.pairs);
   const int gap = min_seed_gap > 0 ? min_seed_gap : k;
@@ -1101,7 +1426,7 @@ int dibella_candidate_pairs_parts(const uint32_t* packed_words, const int64_t* r
     const int lo_bits = 1 + 2 * pbits, hi_bits = 2 * rbits;
     for (int j = 0; j < (lo_bits + 7) / 8 + (hi_bits + 7) / 8; ++j) {
       const int shift = j < (lo_bits + 7) / 8 ? 8 * j : 64 + 8 * (j - (lo_bits + 7) / 8);
-      radix_pass(src, dst, &state->n_keys, shift, hist, hoff, L.tiles, part, &state->status, sms, st);
+      radix_pass(src, dst, &state->n_keys, shift, hist, hoff, L.tiles, part, state, sms, st);
       Key2* tmp = src;
       src = dst;
       dst = tmp;
@@ -1113,7 +1438,7 @@ int dibella_candidate_pairs_parts(const uint32_t* packed_words, const int64_t* r
     unsigned long long* dst = (unsigned long long*)(ws + L.pk1);
     const int passes = (kl.sh_ra + rbits + 7) / 8;
     for (int j = 0; j < passes; ++j) {
-      radix_pass(src, dst, &state->n_keys, 8 * j, hist, hoff, L.tiles, part, &state->status, sms, st);
+      radix_pass(src, dst, &state->n_keys, 8 * j, hist, hoff, L.tiles, part, state, sms, st);
       unsigned long long* tmp = src;
       src = dst;
       dst = tmp;
@@ -1189,8 +1514,7 @@ int dibella_candidate_pairs(const uint32_t* packed_words, const int64_t* read_wo
   const int walk_blocks = sms * 16;
   const int sort_blocks = sms * 8;
   if (n_reads > 0 && L.sort) {
-    // Occurrence keys (code << ib | index), sorted by the code digits only: the
-    // stable passes keep each k-mer's occurrences in index order.
+    // Occurrence keys (mixed code << ib | index), counted in buckets.
     unsigned int* occ_cnt = (unsigned int*)(ws + L.occ_cnt);
     unsigned long long* occ_off = (unsigned long long*)(ws + L.occ_off);
     unsigned long long* ok0 = (unsigned long long*)(ws + L.okeys0);
@@ -1200,17 +1524,14 @@ int dibella_candidate_pairs(const uint32_t* packed_words, const int64_t* read_wo
     occ_count_kernel<<<sms * 4, 256, 0, st>>>(sr, occ_cnt);
     scan_counts(occ_cnt, occ_off, &state->instances, 0, (unsigned long long)n_reads, part, st);
     occ_total_kernel<<<1, 1, 0, st>>>(occ_cnt, occ_off, (long long)n_reads, L.inst, state);
-    extract_kernel<<<walk_blocks, 256, 0, st>>>(sr, occ_off, ib, L.inst, ok0, info);
-    unsigned long long* osrc = ok0;
-    unsigned long long* odst = ok1;
-    for (int j = 0; j < (2 * k + 7) / 8; ++j) {
-      radix_pass(osrc, odst, &state->instances, ib + 8 * j, hist, hoff, L.tiles, part, &state->status, sms, st);
-      unsigned long long* tmp = osrc;
-      osrc = odst;
-      odst = tmp;
-    }
-    run_emit_kernel<<<sms * 8, 256, 0, st>>>(osrc, info, ib, mult_lo, mult_hi, kl, pk0, L.pairs, &state->instances,
-                                             state);
+    // A warp per read, or for few reads several (a set of 124 reads took 37 us with one).
+    const long long need = (n_reads + 7) / 8, share = walk_blocks / need;
+    const dim3 grid((unsigned)(need < walk_blocks ? need : walk_blocks),
+                    (unsigned)(share < 1 ? 1 : (share > 64 ? 64 : share)));
+    extract_kernel<<<grid, 256, 0, st>>>(sr, occ_off, ib, L.inst, ok0, info);
+    if ((e = count_in_buckets(ok0, ok1, info, &state->instances, L.inst, k, ib, mult_lo, mult_hi, kl, pk0, L.pairs,
+                              hist, hoff, part, state, sms, st)) != cudaSuccess)
+      return DIBELLA_ECUDA;
   } else if (n_reads > 0) {
     kmer_walk_kernel<false><<<walk_blocks, 256, 0, st>>>(sr, t, inst, L.inst, mult_lo, mult_hi, state);
     allocate_kernel<<<sms * 8, 256, 0, st>>>(t, L.slots, mult_lo, mult_hi, retained, state);
@@ -1224,11 +1545,12 @@ int dibella_candidate_pairs(const uint32_t* packed_words, const int64_t* read_wo
   unsigned long long* src = pk0;
   unsigned long long* dst = pk1;
   for (int pss = 0; pss < passes; ++pss) {
-    radix_pass(src, dst, &state->n_keys, 8 * pss, hist, hoff, L.tiles, part, &state->status, sms, st);
+    radix_pass(src, dst, &state->n_keys, 8 * pss, hist, hoff, L.tiles, part, state, sms, st);
     unsigned long long* tmp = src;
     src = dst;
     dst = tmp;
   }
+  clear_flags_kernel<<<sms * 8, 256, 0, st>>>(state, flags);
   select_kernel<<<sms * 8, 256, 0, st>>>(src, state, kl, max_seeds, min_seed_gap > 0 ? min_seed_gap : k, flags, sid);
   tile_sum_kernel<<<sort_blocks, kSortThreads, 0, st>>>(flags, state, tsum);
   scan_counts(tsum, toff, &state->n_keys, 2, 0, part, st);
