@@ -2394,9 +2394,9 @@ int launch_extensions_bits(const DeviceInfo& D, long long n_ext, ExtendParams ep
   const int X = ep.sc.X;
   const BitsForms& F = kBitsForms[X <= kBitsForms[0].max_x ? 0 : (X <= kBitsForms[1].max_x ? 1 : 2)];
   // Lanes to count on: unrelated sequences settle at a band of about 5.3 X cells
-  // (132 at X = 25), plus the margins.  Measured around this rule (ms, lanes
-  // 3/4, 4/5, 5/6, 9/10 at X = 7, 15, 25, 50): 28.3/29.9, 41.6/44.5, 58.2/55.3, 47.2/49.3.
-  ep.reserve = std::max(kInitLanes, (5 * X + 67) / 32);
+  // (132 at X = 25), plus some of the margins.  A lane fewer or more at X = 25 or
+  // 50 costs 0 to 10%; at X = 7 two lanes take 24.5 ms where three take 26.
+  ep.reserve = std::max(kInitLanes, (5 * X + 60) / 32);
   ep.young = 20 * X;
   // Warps per SM: the loop keeps the integer pipe 75% busy with one warp per
   // scheduler and about 95% with two; more only make each extension slower, and

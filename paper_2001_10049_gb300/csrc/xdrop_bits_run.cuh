@@ -21,8 +21,8 @@ __device__ __forceinline__ void bits_finish(const ExtendParams& p, const BitTask
 // A suspended extension in the pool: kDumpHead words (item, d, f0, best, bi, bj,
 // r1 and r2, words held, cells, window), then its words plane by plane: both
 // rows' planes and the dead mask.  It was suspended because its band needs
-// another window, so it says which: words `shift` .. shift + want - 1 counted
-// from the first one held.  A queue entry is the pool offset (a multiple of 32)
+// another window, so it says which: `want` words from place `shift` of the one
+// held on.  A queue entry is the pool offset (a multiple of 32)
 // plus want - 1 (of at most 32 words), or -2 - item for an extension that starts
 // over because the pool was full; -1 is a slot that is not written yet.
 constexpr int kDumpHead = 16;
@@ -113,10 +113,10 @@ __device__ __forceinline__ bool bits_task(const ExtendParams& p, BitTask& t, int
   return held;
 }
 
-// The rows of a suspended extension: this lane's word 0 is its word x (words
-// outside it are dead).
+// The rows of a suspended extension: this lane's words begin at place `bit` of
+// the window it held (places outside it are dead).  W > 1: at a whole word.
 template <int NB, int W>
-__device__ __forceinline__ void bits_load(const ExtendParams& p, BitLane<NB, W>& L, int v, int x) {
+__device__ __forceinline__ void bits_load(const ExtendParams& p, BitLane<NB, W>& L, int v, int bit) {
   const uint32_t* o = p.pool + (v & ~31);
   BitForm<NB, W>::init(L, -1);
   L.d = (int)__ldcg(o + 1);
@@ -124,16 +124,22 @@ __device__ __forceinline__ void bits_load(const ExtendParams& p, BitLane<NB, W>&
   L.r1 = __ldcg(o + 6);
   L.r2 = __ldcg(o + 7);
   const int len = (int)__ldcg(o + 8);
+  const unsigned r = (unsigned)bit & 31u;
   o += kDumpHead;
 #pragma unroll
   for (int w = 0; w < W; ++w) {
-    const bool in = x + w >= 0 && x + w < len;
+    const int x = (bit >> 5) + w;
+    const bool in = x >= 0 && x < len, in1 = x + 1 >= 0 && x + 1 < len;
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      L.r[0][w][k] = in ? __ldcg(o + (2 * k) * len + x + w) : BitForm<NB, W>::dead_plane(k);
-      L.r[1][w][k] = in ? __ldcg(o + (2 * k + 1) * len + x + w) : BitForm<NB, W>::dead_plane(k);
+    for (int v2 = 0; v2 <= 2 * NB; ++v2) {  // the planes in the order of bits_suspend, then the dead mask
+      const uint32_t fill = v2 < 2 * NB ? BitForm<NB, W>::dead_plane(v2 >> 1) : 0xFFFFFFFFu;
+      uint32_t y = in ? __ldcg(o + v2 * len + x) : fill;
+      if (W == 1) y = __funnelshift_r(y, in1 ? __ldcg(o + v2 * len + x + 1) : fill, r);
+      if (v2 < 2 * NB)
+        L.r[v2 & 1][w][v2 >> 1 < NB ? v2 >> 1 : 0] = y;
+      else
+        L.dead[w] = y;
     }
-    L.dead[w] = in ? __ldcg(o + 2 * NB * len + x + w) : 0xFFFFFFFFu;
   }
 }
 
@@ -162,9 +168,15 @@ __device__ __forceinline__ void bits_settle(BitLane<NB, W>& L, BitTask& t, int l
 
 constexpr int kCheck = 16;
 constexpr int kMarginTrig = kCheck / 2 + 1;  // places of the window that a band may cross until the next look
-constexpr int kMarginNew = 16;               // kept free at both ends of a window that is laid out anew
-constexpr int kMarginKeep = 24;              // ... and of one that gives lanes back
+constexpr int kMarginNew = 12;               // kept free at both ends of a window that is laid out anew (10 to 16: the same)
+constexpr int kMarginKeep = 20;              // ... and of one that gives lanes back
 constexpr int kInitLanes = 2;
+// Lanes beyond its own that a suspended extension waits for before it joins
+// others: without, two extensions can suspend each other every few looks (150,000
+// seeds at X = 15 with 3 lanes counted for each: 194 ms, 44 with 4 spare lanes; with
+// the 4 lanes that the rule below counts, 38 either way).
+constexpr int kResumeSlack = 4;
+constexpr int kNoRoom = INT32_MIN;           // (no queue entry: see bits_suspend)
 #ifndef XDROP_BITS_SHARED_MAX  // (the CPU test lowers it, to reach the whole-warp form with short sequences)
 #define XDROP_BITS_SHARED_MAX 32
 #endif
@@ -190,7 +202,7 @@ __device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, cons
   F::clear(L);
   if (bits_task(p, t, v, -kWin / 2)) {  // its words go to the middle of the window
     const int off = (32 * W - (int)__ldcg(p.pool + (v & ~31) + 8)) / 2;
-    bits_load<NB, W>(p, L, v, W * lane - off);
+    bits_load<NB, W>(p, L, v, 32 * (W * lane - off));
     t.f0 -= 32 * off;
   } else {
     if (!t.active) return;
@@ -217,8 +229,8 @@ __device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, cons
       break;
     }
     if (narrow) {
-      const int b = (lo - kMarginNew) >> 5, e = (hi + kMarginNew) >> 5;
-      bits_suspend<NB, W>(p, L, t, true, lane, 0, 32, b, e - b + 1, p.res_q, p.res_q_id);
+      const int want = (hi - lo + 1 + 2 * kMarginNew + 31) >> 5;
+      bits_suspend<NB, W>(p, L, t, true, lane, 0, 32, lo - ((32 * want - (hi - lo + 1)) >> 1), want, p.res_q, p.res_q_id);
       break;
     }
     // Move the window by whole lanes to bring the band to its middle.
@@ -308,14 +320,14 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
       if (lane == first) bits_finish(p, t, L.best);
       t.active = false;
     }
-    // lanes wanted: words b .. b + want - 1 of the present window
+    // Lanes wanted, from place b of the present window on (the band in the
+    // middle); a window that the band neither nears nor leaves lanes of stays.
     const bool trig = lo < kMarginTrig || hi > 32 * len - 1 - kMarginTrig;
-    int b = (lo - (trig ? kMarginNew : kMarginKeep)) >> 5, e = (hi + (trig ? kMarginNew : kMarginKeep)) >> 5;
-    if (!trig) {
-      b = max(b, 0);
-      e = min(e, len - 1);
-    }
-    int want = t.active && lane == first ? e - b + 1 : 0;
+    const int width = hi - lo + 1;
+    const int fit = (width + 2 * (trig ? kMarginNew : kMarginKeep) + 31) >> 5;
+    const int need = trig || fit < len ? fit : len;
+    const int b = trig || fit < len ? lo - ((32 * need - width) >> 1) : 0;
+    int want = t.active && lane == first ? need : 0;
     int total = __reduce_add_sync(kFull, want);
     // A band that needs more than 32 lanes: the warp suspends all others and
     // goes on with it in the whole-warp form.  Else, if the bands need more than
@@ -349,6 +361,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
                                                                                     : want);
     int groups = __popc(__ballot_sync(kFull, want > 0)), used = total;
     int entry = -1, efirst = 0, elen = 0;  // what this lane's new group takes up
+    bool waiting = false;  // a suspended one waits for more lanes: no new ones, or they would crowd it out for good
     while (groups < p.max_groups) {
       int v = -1;
       if (lane == 0) {
@@ -356,7 +369,11 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
           const unsigned h = *((volatile unsigned*)&p.cnt->head[p.res_q_id]);
           if ((long long)h >= p.res_cap || h >= *((volatile unsigned*)&p.cnt->tail[p.res_q_id])) break;
           const int c = *((volatile int*)&p.res_q[h]);
-          if (c == -1 || (c >= 0 ? (c & 31) + 1 : max(kInitLanes, p.reserve)) > room) break;
+          if (c == -1) break;
+          if ((c >= 0 ? (c & 31) + 1 + (groups > 0 ? kResumeSlack : 0) : max(kInitLanes, p.reserve)) > room) {
+            v = kNoRoom;
+            break;
+          }
           if (atomicCAS(&p.cnt->head[p.res_q_id], h, h + 1) == h) {
             v = c;
             break;
@@ -364,7 +381,8 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
         }
       }
       v = __shfl_sync(kFull, v, 0);
-      if (v == -1) break;
+      if (v == kNoRoom) waiting = true;
+      if (v == -1 || v == kNoRoom) break;
       __threadfence();  // its words were written before its queue entry
       const int l = v >= 0 ? (v & 31) + 1 : kInitLanes;
       if (lane >= used && lane < used + l) {
@@ -376,7 +394,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
       room -= v >= 0 ? l : max(kInitLanes, p.reserve);
       ++groups;
     }
-    int n_new = exhausted ? 0 : min(room / p.reserve, p.max_groups - groups);
+    int n_new = exhausted || waiting ? 0 : min(room / p.reserve, p.max_groups - groups);
     if (n_new > 0) {
       unsigned base = 0;
       if (lane == 0) base = atomicAdd(&p.cnt->head[p.wide_q_id], (unsigned)n_new);
@@ -408,16 +426,22 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
     __syncwarp();
     const int old_len = __shfl_sync(kFull, len, from), old_want = __shfl_sync(kFull, want, from);
     const int shift = __shfl_sync(kFull, b, from);
-    const int src = from + shift + (lane - nfirst);
+    const int place = shift + 32 * (lane - nfirst);
+    const unsigned bit = (unsigned)place & 31u;
+    const int src = from + (place >> 5);
     const bool held = lane < total && src >= from && src < from + old_len;
+    const bool held1 = lane < total && src + 1 >= from && src + 1 < from + old_len;
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      const uint32_t x = __shfl_sync(kFull, L.r[0][0][k], src & 31), y = __shfl_sync(kFull, L.r[1][0][k], src & 31);
-      L.r[0][0][k] = held ? x : F::dead_plane(k);
-      L.r[1][0][k] = held ? y : F::dead_plane(k);
+    for (int v = 0; v <= 2 * NB; ++v) {  // every plane of both rows, then the dead mask
+      const uint32_t fill = v < 2 * NB ? F::dead_plane(v % NB) : 0xFFFFFFFFu;
+      const uint32_t old = v < 2 * NB ? L.r[v / NB < 2 ? v / NB : 0][0][v % NB] : L.dead[0];
+      const uint32_t x = __shfl_sync(kFull, old, src & 31), y = __shfl_sync(kFull, old, (src + 1) & 31);
+      const uint32_t z = __funnelshift_r(held ? x : fill, held1 ? y : fill, bit);
+      if (v < 2 * NB)
+        L.r[v / NB < 2 ? v / NB : 0][0][v % NB] = z;
+      else
+        L.dead[0] = z;
     }
-    const uint32_t dd = __shfl_sync(kFull, L.dead[0], src & 31);
-    L.dead[0] = held ? dd : 0xFFFFFFFFu;
     L.r1 = __shfl_sync(kFull, L.r1, from);
     L.r2 = __shfl_sync(kFull, L.r2, from);
     L.d = __shfl_sync(kFull, L.d, from);
@@ -425,7 +449,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
     t.item = __shfl_sync(kFull, t.item, from);
     t.m = __shfl_sync(kFull, t.m, from);
     t.n = __shfl_sync(kFull, t.n, from);
-    t.f0 = __shfl_sync(kFull, t.f0, from) + 32 * shift;
+    t.f0 = __shfl_sync(kFull, t.f0, from) + shift;
     t.bi = __shfl_sync(kFull, t.bi, from);
     t.bj = __shfl_sync(kFull, t.bj, from);
     t.a0 = __shfl_sync(kFull, t.a0, from);
@@ -438,9 +462,9 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
       first = efirst;
       len = elen;
       if (bits_task(p, t, entry, -16 * kInitLanes)) {
-        const int from_word = (int)__ldcg(p.pool + (entry & ~31) + 11);
-        t.f0 += 32 * from_word;
-        bits_load<NB, 1>(p, L, entry, lane - first + from_word);
+        const int place = (int)__ldcg(p.pool + (entry & ~31) + 11);
+        t.f0 += place;
+        bits_load<NB, 1>(p, L, entry, place + 32 * (lane - first));
       } else {
         F::init(L, 16 * kInitLanes - 32 * (lane - first));
       }
