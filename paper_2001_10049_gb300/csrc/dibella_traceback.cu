@@ -296,7 +296,7 @@ struct TbBits {
 // whole warp; false if its band outgrew the window.
 template <int NB>
 __device__ bool tb_extend_bits(const TbArgs& p, long long a0, long long b0, int m, int n, const uint32_t (&kx)[NB],
-                               const uint32_t (&ky)[NB], uint32_t* head, uint32_t* moves, TbBits& e) {
+                               uint32_t* head, uint32_t* moves, TbBits& e) {
   using F = BitForm<NB, 1>;
   constexpr int kMargin = 17;  // 32 antidiagonals between looks: at most 16 places either way
   const int lane = threadIdx.x & 31;
@@ -333,9 +333,9 @@ __device__ bool tb_extend_bits(const TbArgs& p, long long a0, long long b0, int 
 #pragma unroll 1
     for (int k = 0; k < 32; k += 2) {
       BitMoves<1> mv;
-      F::template step<true>(L, L.r[0], L.r[1], kx, ky, gm, &mv);
+      F::template step<true, true>(L, L.r[0], L.r[1], kx, gm, &mv);
       record(mv);
-      F::template step<false>(L, L.r[1], L.r[0], kx, ky, gm, &mv);
+      F::template step<false, true>(L, L.r[1], L.r[0], kx, gm, &mv);
       record(mv);
     }
     const uint32_t live[1] = {~L.dead[0]};
@@ -498,7 +498,7 @@ __device__ void tb_walk_bits(const uint32_t* head, const uint32_t* moves, bool d
 // (the caller then takes the extensions one after the other).
 template <int NB>
 __device__ bool tb_extend_both(const TbArgs& p, long long a0, long long b0, int m, int n, const uint32_t (&kx)[NB],
-                               const uint32_t (&ky)[NB], uint32_t* head, uint32_t* moves, uint32_t* end, TbBits& e) {
+                               uint32_t* head, uint32_t* moves, uint32_t* end, TbBits& e) {
   using F = BitForm<NB, 1>;
   constexpr int kMargin = 17, kWin = 512;
   const int lane = threadIdx.x & 31, first = lane & 16, gl = lane & 15;
@@ -532,9 +532,9 @@ __device__ bool tb_extend_both(const TbArgs& p, long long a0, long long b0, int 
 #pragma unroll 1
     for (int k = 0; k < 32; k += 2) {
       BitMoves<1> mv;
-      F::template step<true>(L, L.r[0], L.r[1], kx, ky, gm, &mv);
+      F::template step<true, true>(L, L.r[0], L.r[1], kx, gm, &mv);
       record(mv);
-      F::template step<false>(L, L.r[1], L.r[0], kx, ky, gm, &mv);
+      F::template step<false, true>(L, L.r[1], L.r[0], kx, gm, &mv);
       record(mv);
     }
     const uint32_t live[1] = {~L.dead[0]};
@@ -596,8 +596,8 @@ __device__ bool tb_seed_bits(const TbArgs& p, long long t, char* scratch, const 
                              long long lenB) {
   const int lane = threadIdx.x & 31;
   const int k = p.k;
-  uint32_t kx[NB], ky[NB];
-  bits_threshold<NB>(p.X, kx, ky);
+  uint32_t kx[NB];
+  bits_threshold<NB>(p.X, kx);
   uint32_t* head = (uint32_t*)scratch;
   uint32_t* moves = head + ((2ll * p.max_len + 5) & ~1ll);
   const long long fA = p.word_offsets[pr.read_a] * 16, rA = fA + tb_copy_words(lenA) * 16;
@@ -629,7 +629,7 @@ __device__ bool tb_seed_bits(const TbArgs& p, long long t, char* scratch, const 
   uint32_t* own = head + (rt ? lm + ln + 1 : 0);
   uint32_t* end = (uint32_t*)(scratch + 12ll * (p.max_len + 2) + 4 * p.moves_words);
   end -= (end - head) & 1;
-  if (tb_extend_both<NB>(p, rt ? ra : la, rt ? rb : lb, rt ? rm : lm, rt ? rn : ln, kx, ky, own, moves, end, e)) {
+  if (tb_extend_both<NB>(p, rt ? ra : la, rt ? rb : lb, rt ? rm : lm, rt ? rn : ln, kx, own, moves, end, e)) {
     const int d = e.i_end + e.j_end;
     TbWarpRuns both{rt ? own + d : ops, rt ? (long long)d : (long long)p.ops_per_seed, rt ? -1 : 1, (lane & 15) == 0,
                     0, 0, 0};
@@ -645,14 +645,14 @@ __device__ bool tb_seed_bits(const TbArgs& p, long long t, char* scratch, const 
     back_last = head + (lm + ln + 1) + er.i_end + er.j_end - back.n + 1;
     seed_columns();
   } else {
-    if (!tb_extend_bits<NB>(p, la, lb, lm, ln, kx, ky, head, moves, el)) return false;
+    if (!tb_extend_bits<NB>(p, la, lb, lm, ln, kx, head, moves, el)) return false;
     ok = el.recorded;
     if (ok) {
       tb_walk_bits<32>(head, moves, false, el.i_end, el.j_end, el.best_off, runs);
       seed_columns();
     }
     __syncwarp();  // the left walk has read the records before the right extension rewrites them
-    if (!tb_extend_bits<NB>(p, ra, rb, rm, rn, kx, ky, head, moves, er)) return false;
+    if (!tb_extend_bits<NB>(p, ra, rb, rm, rn, kx, head, moves, er)) return false;
     if (ok) ok = er.recorded;
     if (ok) {
       const int d = er.i_end + er.j_end;

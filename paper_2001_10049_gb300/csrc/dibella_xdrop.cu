@@ -1895,8 +1895,8 @@ std::mutex g_dev_mu;
 DeviceInfo g_dev[64];
 
 // The bit-sliced form by the planes that X needs (kD = 2^planes - 2 has to stay
-// above every live value: X <= 2^planes - 5).  Each plane more costs about 9% of
-// an antidiagonal (107 warp instructions at 5 planes).  Beyond X = 59 the int16
+// above every live value: X <= 2^planes - 5).  Each plane more costs about 10% of
+// an antidiagonal (about 97 warp instructions at 5 planes).  Beyond X = 59 the int16
 // forms run: a seventh plane would take X to 123, where no workload goes.
 using BitsKernel = void (*)(ExtendParams);
 struct BitsForms {

@@ -44,13 +44,16 @@
 // whose band no longer fits is handed on.
 
 // What bounds it: the integer pipe.  An antidiagonal of a warp (5 planes, one word
-// a lane) is 107 instructions, 89 of them on that pipe at one per two cycles a
-// scheduler; a warp alone takes 234 cycles for it, and two warps a scheduler keep
-// the pipe about 95% busy.  Memory traffic is one word of bases per lane and 32
-// antidiagonals.  Batches in ms, this form / the int16 forms: E. coli-sized reads
-// at X = 7 (400,000 seeds) 28.2 / 147 and at X = 25 (150,000) 53.5 / 365, the
-// repeat-rich reads at X = 15 (150,000) 44 / 310, reads of 500 b to 100 kb at
-// X = 50 (12,000) 73 / 380, one seed of 4 kb reads 0.16 / 1.2.
+// a lane) is about 97 instructions, 79 of them on that pipe at one per two cycles a
+// scheduler; two warps a scheduler keep the pipe 81 to 87% busy (counters at X = 7
+// and 25).  Memory traffic is one word of bases per lane and 32 antidiagonals.
+// Carrying r1 into the comparison with X instead of selecting X - r1, leaving the
+// validity planes out of loops that stay inside the matrix, and one shift for the
+// mask below the highest bit took it there from 107 and 89 (E. coli-sized batches
+// 6 to 8% faster).  Batches in ms, this form / the int16 forms: E. coli-sized reads
+// at X = 7 (400,000 seeds) 22.6 / 147 and at X = 25 (150,000) 46.6 / 369, the
+// repeat-rich reads at X = 15 (150,000, on the device) 35.7 / 310, reads of 500 b
+// to 100 kb at X = 50 (12,000) 55 to 71 / 380, one seed of 4 kb reads 0.16 / 1.2.
 
 template <int LUT>
 __device__ __forceinline__ uint32_t lop3(uint32_t a, uint32_t b, uint32_t c) {
@@ -71,6 +74,17 @@ __host__ __device__ constexpr int lnot(int x) { return ~x & 0xFF; }
 // x >> n and x << n with n clamped at 32 (PTX shift semantics).
 __device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t n) { return __funnelshift_rc(x, 0u, n); }
 __device__ __forceinline__ uint32_t shl_clamp(uint32_t x, uint32_t n) { return __funnelshift_lc(0u, x, n); }
+
+// All ones up to the highest set bit of x, 0 for x = 0.
+__device__ __forceinline__ uint32_t ones_to_highest(uint32_t x) {
+#ifdef XDROP_BITS_EMULATE
+  return x ? 0xFFFFFFFFu >> __clz((int)x) : 0u;
+#else
+  uint32_t r;  // the shift is the leading zeros, or 2^32 - 1 for x = 0 (shr clamps at 32)
+  asm("{ .reg .u32 t;\n bfind.shiftamt.u32 t, %1;\n shr.u32 %0, 0xFFFFFFFF, t; }" : "=r"(r) : "r"(x));
+  return r;
+#endif
+}
 
 // 16 bases (base q at bits 2q) to their low bits (bits 0-15) and high bits (16-31).
 __device__ __forceinline__ uint32_t split_planes(uint32_t x) {
@@ -149,14 +163,15 @@ struct BitForm {
   using Lane = BitLane<NB, W>;
 
   // One antidiagonal: row P (d-1) and row Q (d-2, overwritten with d).
-  // kx[k] / ky[k]: bit k of X / X - 1 as a mask.  With `moves` the cells' band
+  // kx[k]: bit k of X as a mask.  CLIP: the window or what enters it reaches
+  // beyond the matrix (else the validity planes are all ones and stay so).  With `moves` the cells' band
   // and the move that gave each its value (equal values: the diagonal first, then
   // the step in A, then the step in B') as two planes: 00 diagonal, 01 diagonal
   // on equal bases, 10 A, 11 B'.
-  template <bool E>
+  template <bool E, bool CLIP>
   __device__ static __forceinline__ void step(Lane& L, uint32_t (&P)[W][NB], uint32_t (&Q)[W][NB],
-                                              const uint32_t (&kx)[NB], const uint32_t (&ky)[NB],
-                                              const GroupMasks& gm, BitMoves<W>* moves = nullptr) {
+                                              const uint32_t (&kx)[NB], const GroupMasks& gm,
+                                              BitMoves<W>* moves = nullptr) {
     // Neighbour lane's word for the one-cell shift (E: from above, O: from
     // below).  At a group's ends the plane bits that come in are whatever the
     // neighbour group holds: those places are outside every band.
@@ -172,21 +187,21 @@ struct BitForm {
       for (int w = 0; w < W; ++w) {
         L.a0[w] = __funnelshift_r(L.a0[w], w + 1 < W ? L.a0[w + 1 < W ? w + 1 : w] : L.fa0, 1);
         L.a1[w] = __funnelshift_r(L.a1[w], w + 1 < W ? L.a1[w + 1 < W ? w + 1 : w] : L.fa1, 1);
-        L.va[w] = __funnelshift_r(L.va[w], w + 1 < W ? L.va[w + 1 < W ? w + 1 : w] : L.fva, 1);
+        if (CLIP) L.va[w] = __funnelshift_r(L.va[w], w + 1 < W ? L.va[w + 1 < W ? w + 1 : w] : L.fva, 1);
       }
       L.fa0 >>= 1;
       L.fa1 >>= 1;
-      L.fva >>= 1;
+      if (CLIP) L.fva >>= 1;
     } else {
 #pragma unroll
       for (int w = W - 1; w >= 0; --w) {
         L.b0[w] = __funnelshift_l(w > 0 ? L.b0[w > 0 ? w - 1 : 0] : L.fb0, L.b0[w], 1);
         L.b1[w] = __funnelshift_l(w > 0 ? L.b1[w > 0 ? w - 1 : 0] : L.fb1, L.b1[w], 1);
-        L.vb[w] = __funnelshift_l(w > 0 ? L.vb[w > 0 ? w - 1 : 0] : L.fvb, L.vb[w], 1);
+        if (CLIP) L.vb[w] = __funnelshift_l(w > 0 ? L.vb[w > 0 ? w - 1 : 0] : L.fvb, L.vb[w], 1);
       }
       L.fb0 <<= 1;
       L.fb1 <<= 1;
-      L.fvb <<= 1;
+      if (CLIP) L.fvb <<= 1;
     }
     // Band: the live mask widened by a cell, filled between its ends.
     uint32_t band[W];
@@ -207,20 +222,17 @@ struct BitForm {
       uint32_t acc = above;
 #pragma unroll
       for (int w = W - 1; w >= 0; --w) {
-        dn[w] = acc | shr_clamp(0xFFFFFFFFu, (uint32_t)__clz((int)x[w]));
+        dn[w] = acc | ones_to_highest(x[w]);
         if (w > 0) acc |= x[w] ? 0xFFFFFFFFu : 0u;
       }
 #pragma unroll
       for (int w = 0; w < W; ++w) {
         const uint32_t u = up | x[w] | (0u - x[w]);
         if (w + 1 < W) up |= x[w] ? 0xFFFFFFFFu : 0u;
-        band[w] = u & dn[w] & L.va[w] & L.vb[w];
+        band[w] = CLIP ? u & dn[w] & L.va[w] & L.vb[w] : u & dn[w];
         L.cells += __popc(band[w]);
       }
     }
-    uint32_t kc[NB];  // bits of X - r1
-#pragma unroll
-    for (int k = 0; k < NB; ++k) kc[k] = lop3<(kLA & kLB) | (lnot(kLA) & kLC)>(L.r1, ky[k], kx[k]);
     uint32_t imp[W], any_imp = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
@@ -262,11 +274,12 @@ struct BitForm {
         moves->hi[w] = gap;
         moves->lo[w] = lop3<(kLA & kLB) | (lnot(kLA) & kLC)>(gap, from_b, eq);
       }
-      uint32_t m[NB], gt = 0;
+      // gt: m > X - r1, i.e. m > X, or m = X and r1 (r1 carried in)
+      uint32_t m[NB], gt = L.r1;
 #pragma unroll
       for (int k = 0; k < NB; ++k) {
         m[k] = lop3<(kLA & kLB) | (lnot(kLA) & kLC)>(gap, g[k], q[k]);
-        gt = k == 0 ? (m[0] & ~kc[0]) : lop3<(kLA & lnot(kLB)) | (lnot(kLA ^ kLB) & kLC)>(m[k], kc[k], gt);
+        gt = lop3<(kLA & lnot(kLB)) | (lnot(kLA ^ kLB) & kLC)>(m[k], kx[k], gt);
       }
       const uint32_t dd = lop3<(kLA & lnot(kLB)) | lnot(kLC)>(gt, bor, band[w]);
       imp[w] = lop3<kLA & kLB & lnot(kLC)>(bor, band[w], L.r1);
@@ -344,6 +357,25 @@ struct BitForm {
     L.fvb = shl_clamp(0xFFFFFFFFu, (uint32_t)min(max(32 - (n - y), 0), 32));
   }
 
+  // Whether the window or what enters it over the next 32 steps reaches beyond
+  // the matrix in this lane (after load_window and load_feed).
+  __device__ static __forceinline__ bool clipped(const Lane& L) {
+    uint32_t all = (L.fva | 0xFFFF0000u) & (L.fvb | 0x0000FFFFu);
+#pragma unroll
+    for (int w = 0; w < W; ++w) all &= L.va[w] & L.vb[w];
+    return all != 0xFFFFFFFFu;
+  }
+
+  // N antidiagonals, an even number, from a row at an even d.
+  template <int N, bool CLIP>
+  __device__ static __forceinline__ void steps(Lane& L, const uint32_t (&kx)[NB], const GroupMasks& gm) {
+#pragma unroll 1
+    for (int k = 0; k < N; k += 2) {
+      step<true, CLIP>(L, L.r[0], L.r[1], kx, gm);
+      step<false, CLIP>(L, L.r[1], L.r[0], kx, gm);
+    }
+  }
+
   // Row d = 0 (cell (0,0), drop 0) at the window place that is bit `bit` of
   // this lane (in [0, 32 W), or outside it); nothing before it.  The lane's
   // sequences are not touched.
@@ -380,10 +412,7 @@ struct BitForm {
 };
 
 template <int NB>
-__device__ __forceinline__ void bits_threshold(int X, uint32_t (&kx)[NB], uint32_t (&ky)[NB]) {
+__device__ __forceinline__ void bits_threshold(int X, uint32_t (&kx)[NB]) {
 #pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    kx[k] = (X >> k) & 1 ? 0xFFFFFFFFu : 0u;
-    ky[k] = ((X - 1) >> k) & 1 ? 0xFFFFFFFFu : 0u;
-  }
+  for (int k = 0; k < NB; ++k) kx[k] = (X >> k) & 1 ? 0xFFFFFFFFu : 0u;
 }

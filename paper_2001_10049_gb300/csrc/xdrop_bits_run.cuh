@@ -189,8 +189,7 @@ constexpr int kNarrowAgain = 24 * kSharedMax;      // live cells below which the
 // outgrows this form too goes to esc_q (from W = 4 on: to the forms that hold
 // scores, from the start).
 template <int NB, int W, bool BACK>
-__device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, const uint32_t (&kx)[NB],
-                                              const uint32_t (&ky)[NB]) {
+__device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, const uint32_t (&kx)[NB]) {
   using F = BitForm<NB, W>;
   constexpr int kWin = 32 * 32 * W;
   constexpr int kMargin = 17;  // 32 antidiagonals between looks: at most 16 places either way
@@ -211,11 +210,7 @@ __device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, cons
   F::load_window(L, words, t.a0, t.b0, t.m, t.n, t.window(L.d) + 32 * W * lane, L.d);
   for (;;) {
     F::load_feed(L, words, t.a0, t.b0, t.m, t.n, t.window(L.d) + 32 * W * lane, L.d);
-#pragma unroll 1
-    for (int k = 0; k < 32; k += 2) {
-      F::template step<true>(L, L.r[0], L.r[1], kx, ky, gm);
-      F::template step<false>(L, L.r[1], L.r[0], kx, ky, gm);
-    }
+    F::template steps<32, true>(L, kx, gm);
     uint32_t live[W];
 #pragma unroll
     for (int w = 0; w < W; ++w) live[w] = ~L.dead[w];
@@ -269,13 +264,13 @@ __device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, cons
 // The extensions of the queue one by one (persistent).
 template <int NB, int W>
 __device__ __forceinline__ void bits_warp_run(const ExtendParams& p) {
-  uint32_t kx[NB], ky[NB];
-  bits_threshold<NB>(p.sc.X, kx, ky);
+  uint32_t kx[NB];
+  bits_threshold<NB>(p.sc.X, kx);
   const unsigned tail = *((volatile unsigned*)&p.cnt->tail[p.wide_q_id]);
   for (;;) {
     const unsigned q = pop_warp(p.cnt, p.wide_q_id);
     if (q >= tail) break;
-    bits_warp_one<NB, W, false>(p, p.wide_q[q], kx, ky);
+    bits_warp_one<NB, W, false>(p, p.wide_q[q], kx);
   }
 }
 
@@ -297,8 +292,8 @@ template <int NB>
 __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map) {
   using F = BitForm<NB, 1>;
   const int lane = threadIdx.x & 31;
-  uint32_t kx[NB], ky[NB];
-  bits_threshold<NB>(p.sc.X, kx, ky);
+  uint32_t kx[NB];
+  bits_threshold<NB>(p.sc.X, kx);
   const unsigned tail = *((volatile unsigned*)&p.cnt->tail[p.wide_q_id]);
   const uint32_t* __restrict__ words = p.words;
   typename F::Lane L;
@@ -346,7 +341,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
       total = __reduce_add_sync(kFull, want);
     }
     if (alone != -1) {
-      bits_warp_one<NB, 2, true>(p, alone, kx, ky);
+      bits_warp_one<NB, 2, true>(p, alone, kx);
       t.active = false;
       F::clear(L);
       first = lane;
@@ -481,14 +476,15 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
     const uint32_t near_end = (gm.end_lo & ((1u << kMarginTrig) - 1u)) | (gm.end_hi & ~((1u << (32 - kMarginTrig)) - 1u));
     for (;;) {
       if (t.active) F::load_feed(L, words, t.a0, t.b0, t.m, t.n, t.window(L.d) + 32 * (lane - first), L.d);
+      // (a lane without work is never clipped: its planes stay 0 and its band empty)
+      const bool clip = __any_sync(kFull, t.active && F::clipped(L));
       bool look = false;
 #pragma unroll 1
       for (int h = 0; h < 32 && !look; h += kCheck) {
-#pragma unroll 1
-        for (int k = 0; k < kCheck; k += 2) {
-          F::template step<true>(L, L.r[0], L.r[1], kx, ky, gm);
-          F::template step<false>(L, L.r[1], L.r[0], kx, ky, gm);
-        }
+        if (clip)
+          F::template steps<kCheck, true>(L, kx, gm);
+        else
+          F::template steps<kCheck, false>(L, kx, gm);
         const uint32_t any = __ballot_sync(kFull, L.dead[0] != 0xFFFFFFFFu);
         look = __any_sync(kFull, t.active && ((any & gm.grp) == 0 || (~L.dead[0] & near_end) != 0));
       }
