@@ -611,14 +611,23 @@ def mode_stream(args):
 # Algorithmic DRAM bytes of candidate generation.  Sort-based count (code and
 # occurrence index share one 64-bit key): per k-mer occurrence, the 2-bit
 # sequence (0.5 B), the key and its (read, position, orientation) word written
-# (16 B), each 8-bit pass over the code digits reading the key for the
-# histogram and reading and writing it in the scatter (24 B), and the run walk
-# reading the key and gathering the word (16 B).  Hash-table count (wider
+# (16 B), each 8-bit pass over the bucket bits of the mixed code (16 bits, for
+# buckets of about 2,048 occurrences) reading the key for the histogram and
+# reading and writing it in the scatter (24 B), the bucket starts (8 B) and the
+# buckets (8 B) reading it; the words of the retained occurrences are few.
+# Hash-table count (wider
 # keys): two walks each touching one 8-byte table key and one 4-byte counter,
 # plus the sequence (24.5 B).  Per occurrence pair: the 8-byte key written,
 # 24 B per pass of its sort, read by selection and compaction (16 B).
-def cand_bytes_per_occ(sort_count: bool, k: int) -> float:
-    return 32.5 + 24 * ((2 * k + 7) // 8) if sort_count else 24.5
+def cand_bytes_per_occ(sort_count: bool, k: int, n_bases: int) -> float:
+    return 32.5 + 24 * cand_bucket_passes(k, n_bases) if sort_count else 24.5
+
+
+def cand_bucket_passes(k: int, n_bases: int) -> int:
+    bits = 0
+    while bits < min(16, 2 * k) and (n_bases >> bits) > 2048:
+        bits += 1
+    return (bits + 7) // 8
 
 
 def cand_bytes_per_pair(passes: int) -> int:
@@ -626,9 +635,8 @@ def cand_bytes_per_pair(passes: int) -> int:
 
 
 # DRAM bytes of one call (every kernel of the call, from one ncu capture) for
-# kernels unchanged since that capture; none is current: the radix passes moved
-# from 16,384- to 8,192-key tiles after the last DRAM capture (25,658,249,318 B
-# per call then), and the current launch list
+# kernels unchanged since that capture; none is current: the counting kernels
+# changed after the last DRAM capture, and the current launch list
 # (profiles/candidate_pairs_c2_ecoli_launch_list.md) holds durations only.
 CAND_NCU_TRAFFIC = {}
 
@@ -683,7 +691,7 @@ def mode_candidates(args):
     pbits = max(1, int(store.max_len).bit_length())
     passes = (2 * rbits + 2 * pbits + 1 + 7) // 8
     sort_count = 2 * p["k"] + max(1, int(store.n_bases).bit_length()) <= 64
-    per_occ = cand_bytes_per_occ(sort_count, p["k"])
+    per_occ = cand_bytes_per_occ(sort_count, p["k"], store.n_bases)
     alg = per_occ * int(c[2]) + cand_bytes_per_pair(passes) * int(c[4])
     n_cand = int(c[1])
     cpu = None
@@ -711,8 +719,9 @@ def mode_candidates(args):
         "roofline": {"bound": "hbm", "achieved": alg / (ms * 1e-3) / 1e9, "peak": pk["hbm_gbs"], "unit": "GB/s",
                      "frac": alg / (ms * 1e-3) / 1e9 / pk["hbm_gbs"],
                      "traffic": CAND_NCU_TRAFFIC.get(w.name),
-                     "kernel": ("whole call (occurrence keys, %d radix passes by code, run walk, %d radix passes"
-                                " of the pairs, select, compact)" % ((2 * p["k"] + 7) // 8, passes)) if sort_count
+                     "kernel": ("whole call (occurrence keys, %d radix passes by bucket, bucket counts, %d radix passes"
+                                " of the pairs, select, compact)" % (cand_bucket_passes(p["k"], store.n_bases),
+                                                                     passes)) if sort_count
                      else "whole call (count, allocate, fill, emit, %d radix passes, select, compact)" % passes,
                      "peak_source": "%s hbm_gbs" % pk_kind,
                      "bytes_model": "%.1f B per k-mer occurrence + %d B per occurrence pair"
@@ -977,7 +986,9 @@ def main():
     for X in XD:
         phase[X] = np.concatenate([phase[X][:1], [phase[X][1] + phase[X][2]], phase[X][3:]])
     batch_ms = {X: float(np.mean([ms for (x, ms, _) in log if x == X])) for X in XD}
-    launch_cells = {X: {"narrow form": (1, counters[X]["cells_narrow"]),
+    # without a schedule every extension runs in the bit-sliced form, whose one launch stands as the narrow form's
+    first_form = "narrow form" if sched is not None else "bit-sliced form, shared lanes"
+    launch_cells = {X: {first_form: (1, counters[X]["cells_narrow"]),
                         "wide form, first launch": (2, counters[X]["cells_wide"] - counters[X]["cells_wide_esc"]
                                                      - counters[X]["cells_ladder"]),
                         "mid form on the narrow escalations": (3, counters[X]["cells_mid"]),
@@ -1033,6 +1044,9 @@ def main():
                      "peak_source": "%d SMs x %d INT32 lanes x %.0f MHz (%s sm_max_mhz)"
                                     % (sm_count, INT32_LANES_PER_SM, pk.get("sm_max_mhz", 2070.0), pk_kind),
                      "ops_per_cell": OPS_PER_CELL,
+                     "ops_note": "8 per cell is the convention of a cell-by-cell DP; the bit-sliced form issues about "
+                                 "3 lane instructions a cell of its windows (32 cells to a logic instruction), so the "
+                                 "fractions compare it with such a DP; its integer pipe is 81 to 87% busy",
                      "peak_measured": cell_peak, "frac_measured": achieved / cell_peak,
                      "peak_measured_class": "int32 DP cell, 8 ops (compare, select, add; max, add; max; "
                                             "compare, select), full grid of independent chains",

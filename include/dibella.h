@@ -464,7 +464,9 @@ int dibella_xdrop_traceback(const uint32_t* packed_words, const int64_t* read_wo
  * dibella_xdrop_batch; results hold the last run's output.  Synchronises
  * `stream`; refused (EINVAL) while `stream` is capturing.  *best_ms_out and
  * *n_tried_out (either may be NULL) receive the winner's time and the number
- * of schedules timed.  The paper has no tuner; its Sec. 9 names the cost
+ * of schedules timed.  (Every one of them is an explicit schedule: where the
+ * bit-sliced form applies, a call without a schedule is faster.)
+ * The paper has no tuner; its Sec. 9 names the cost
  * differences (read length, X-drop early exit) this one adapts to. */
 int dibella_autotune(const uint32_t* packed_words, const int64_t* read_word_offsets,
                      const int32_t* read_lengths, int64_t n_reads, const dibella_pair_t* pairs,
