@@ -1046,7 +1046,7 @@ def main():
                      "ops_per_cell": OPS_PER_CELL,
                      "ops_note": "8 per cell is the convention of a cell-by-cell DP; the bit-sliced form issues about "
                                  "3 lane instructions a cell of its windows (32 cells to a logic instruction), so the "
-                                 "fractions compare it with such a DP; its integer pipe is 81 to 87% busy",
+                                 "fractions compare it with such a DP; its integer pipe is 85 to 92% busy",
                      "peak_measured": cell_peak, "frac_measured": achieved / cell_peak,
                      "peak_measured_class": "int32 DP cell, 8 ops (compare, select, add; max, add; max; "
                                             "compare, select), full grid of independent chains",

@@ -2399,7 +2399,7 @@ int launch_extensions_bits(const DeviceInfo& D, long long n_ext, ExtendParams ep
   ep.reserve = std::max(kInitLanes, (5 * X + 60) / 32);
   ep.young = 20 * X;
   // Warps per SM: the loop keeps the integer pipe 75% busy with one warp per
-  // scheduler and about 95% with two; more only make each extension slower, and
+  // scheduler and 85 to 92% with two; more only make each extension slower, and
   // the longest one ends the launch (E. coli-sized reads at X = 25, 300,000
   // extensions: 70 / 55 / 74 ms with 1 / 2 / 3 blocks).  Small batches take one,
   // and spread out over all warps: each extension runs fastest alone.

@@ -45,8 +45,8 @@
 
 // What bounds it: the integer pipe.  An antidiagonal of a warp (5 planes, one word
 // a lane) is about 97 instructions, 79 of them on that pipe at one per two cycles a
-// scheduler; two warps a scheduler keep the pipe 81 to 87% busy (counters at X = 7
-// and 25).  Memory traffic is one word of bases per lane and 32 antidiagonals.
+// scheduler; two warps a scheduler keep the pipe 85 to 92% busy (counters at X = 7,
+// 25 and 50).  Memory traffic is one word of bases per lane and 32 antidiagonals.
 // Carrying r1 into the comparison with X instead of selecting X - r1, leaving the
 // validity planes out of loops that stay inside the matrix, and one shift for the
 // mask below the highest bit took it there from 107 and 89 (E. coli-sized batches
