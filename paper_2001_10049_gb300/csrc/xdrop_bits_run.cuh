@@ -9,6 +9,7 @@ struct BitTask {
   int bi, bj;    // cell of the best score
   long long a0, b0, cells;
   bool active;
+  int restarts;  // times it has started over in the shared-lane form, as the pool was full
   __device__ __forceinline__ int window(int d) const { return f0 + ((d + 1) >> 1); }
 };
 
@@ -25,7 +26,20 @@ __device__ __forceinline__ void bits_finish(const ExtendParams& p, const BitTask
 // held on.  A queue entry is the pool offset (a multiple of 32)
 // plus want - 1 (of at most 32 words), or -2 - item for an extension that starts
 // over because the pool was full; -1 is a slot that is not written yet.
+//
+// The pool is not given back within a launch, and once a request has found it
+// full it stays full.  From then on what is suspended starts over, so that has to
+// end: an extension starts over at most kMaxRestarts times in the shared-lane form
+// (counted in its result's status until then) and goes on to the whole-warp launch,
+// and the whole-warp form keeps one whose band has become narrow instead of handing
+// it back.  (Bounded by the queue's slots alone, 6,000 bases of AC against as many
+// of A at X = 25 were started 202 times with 100 slots.)
 constexpr int kDumpHead = 16;
+// (1.7 M E. coli-sized seeds at X = 25, whose 734,000 suspensions run out of pool:
+// 1,098 / 987 / 950 ms with 2 / 4 / 8 where no limit took 946, and 939 with 16 where
+// no limit took 938.  What is passed on has a warp of 4 words a lane to itself:
+// 4.9 / 1.4 / 0.15 / 0.003% of the cells, in 335 / 95 / 13 / 6 ms.)
+constexpr int kMaxRestarts = 16;
 template <int NB>
 __device__ __forceinline__ unsigned dump_words(int len) {
   return (unsigned)(kDumpHead + (2 * NB + 1) * len + 31) & ~31u;
@@ -33,11 +47,12 @@ __device__ __forceinline__ unsigned dump_words(int len) {
 
 // Writes the extension of lanes first .. first + len - 1 (W words each) to the
 // pool and its entry to `queue` (null: none).  Every lane of the warp calls it;
-// `mine` says whose group it is.  Returns the entry.
+// `mine` says whose group it is.  Returns the entry; with `keep`, -1 and nothing
+// done if the pool is full.
 template <int NB, int W>
 __device__ __forceinline__ int bits_suspend(const ExtendParams& p, const BitLane<NB, W>& L, const BitTask& t, bool mine,
                                              int lane, int first, int len, int shift, int want, int* queue,
-                                             int q_id) {
+                                             int q_id, bool keep = false) {
   const bool leader = mine && lane == first;
   const unsigned size = dump_words<NB>(W * len);
   int off = -1;
@@ -46,6 +61,7 @@ __device__ __forceinline__ int bits_suspend(const ExtendParams& p, const BitLane
     if (at + size <= p.pool_words) off = (int)at;
   }
   off = __shfl_sync(kFull, off, first);
+  if (keep && off < 0) return -1;
   if (mine && off >= 0) {
     uint32_t* o = p.pool + off;
     if (leader) {
@@ -77,7 +93,18 @@ __device__ __forceinline__ int bits_suspend(const ExtendParams& p, const BitLane
   __syncwarp();
   const int entry = off >= 0 ? off + min(want, 32) - 1 : -2 - t.item;
   if (leader) {
-    if (off < 0) atomicAdd(&p.cnt->cells[7], (unsigned long long)t.cells);
+    if (off < 0) {
+      atomicAdd(&p.cnt->cells[7], (unsigned long long)t.cells);
+      if (queue == p.res_q) {
+        if (t.restarts < kMaxRestarts) {
+          p.ext[t.item].status = t.restarts + 1;
+          __threadfence();
+        } else {
+          queue = p.esc_q;
+          q_id = p.esc_q_id;
+        }
+      }
+    }
     atomicAdd(&p.cnt->stat[p.bits_esc_stat], 1u);
   }
   if (leader && queue != nullptr) {
@@ -99,6 +126,7 @@ __device__ __forceinline__ bool bits_task(const ExtendParams& p, BitTask& t, int
   const bool held = v >= 0;
   const uint32_t* o = p.pool + (v & ~31);
   t.item = held ? (int)__ldcg(o) : -2 - v;
+  t.restarts = 0;
   t.active = DIBELLA_IN_BOUNDS(t.item, p.q_cap, 3);  // (debug build: a bad item is dropped)
   if (!t.active) return false;
   const Item it = p.items[t.item];
@@ -185,9 +213,9 @@ constexpr int kNarrowAgain = 24 * kSharedMax;      // live cells below which the
 
 // Whole-warp form: the extension of queue entry v by all 32 lanes, W words
 // each, for a band that outgrows one word a lane.  With BACK it is suspended to
-// the shared-lane form again once its band has become narrow; a band that
-// outgrows this form too goes to esc_q (from W = 4 on: to the forms that hold
-// scores, from the start).
+// the shared-lane form again once its band has become narrow, while the pool has
+// room; a band that outgrows this form too goes to esc_q (from W = 4 on: to the
+// forms that hold scores, from the start).
 template <int NB, int W, bool BACK>
 __device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, const uint32_t (&kx)[NB]) {
   using F = BitForm<NB, W>;
@@ -208,6 +236,7 @@ __device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, cons
     F::init(L, kWin / 2 - 32 * W * lane);
   }
   F::load_window(L, words, t.a0, t.b0, t.m, t.n, t.window(L.d) + 32 * W * lane, L.d);
+  bool back = BACK;
   for (;;) {
     F::load_feed(L, words, t.a0, t.b0, t.m, t.n, t.window(L.d) + 32 * W * lane, L.d);
     F::template steps<32, true>(L, kx, gm);
@@ -216,8 +245,9 @@ __device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, cons
     for (int w = 0; w < W; ++w) live[w] = ~L.dead[w];
     int lo, hi;
     group_ends<W>(live, lane, 0, kFull, lo, hi);
-    const bool narrow = BACK && lo >= 0 && hi - lo < kNarrowAgain;
-    if (lo >= kMargin && hi <= kWin - 1 - kMargin && !narrow) continue;
+    const bool narrow = back && lo >= 0 && hi - lo < kNarrowAgain;
+    const bool inside = lo >= kMargin && hi <= kWin - 1 - kMargin;
+    if (inside && !narrow) continue;
     bits_settle<NB, W>(L, t, lane, 0, 32, gm);
     if (lo < 0) {  // ended
       if (lane == 0) bits_finish(p, t, L.best);
@@ -225,8 +255,11 @@ __device__ __forceinline__ void bits_warp_one(const ExtendParams& p, int v, cons
     }
     if (narrow) {
       const int want = (hi - lo + 1 + 2 * kMarginNew + 31) >> 5;
-      bits_suspend<NB, W>(p, L, t, true, lane, 0, 32, lo - ((32 * want - (hi - lo + 1)) >> 1), want, p.res_q, p.res_q_id);
-      break;
+      if (bits_suspend<NB, W>(p, L, t, true, lane, 0, 32, lo - ((32 * want - (hi - lo + 1)) >> 1), want, p.res_q,
+                              p.res_q_id, true) != -1)
+        break;
+      back = false;
+      if (inside) continue;
     }
     // Move the window by whole lanes to bring the band to its middle.
     const int by = ((lo + hi) / 2 - kWin / 2 + (lo < kMargin ? -16 * W : 16 * W)) / (32 * W);
@@ -301,6 +334,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
   BitTask t;
   t.item = t.m = t.n = t.f0 = t.bi = t.bj = 0;
   t.a0 = t.b0 = t.cells = 0;
+  t.restarts = 0;
   t.active = false;
   int first = lane, len = 1;  // this lane's group; a lane without work is a group of its own
   GroupMasks gm = group_masks(lane, first, len);
@@ -356,6 +390,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
                                                                                     : want);
     int groups = __popc(__ballot_sync(kFull, want > 0)), used = total;
     int entry = -1, efirst = 0, elen = 0;  // what this lane's new group takes up
+    bool over = false;
     bool waiting = false;  // a suspended one waits for more lanes: no new ones, or they would crowd it out for good
     while (groups < p.max_groups) {
       int v = -1;
@@ -382,6 +417,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
       const int l = v >= 0 ? (v & 31) + 1 : kInitLanes;
       if (lane >= used && lane < used + l) {
         entry = v;
+        over = v < 0;
         efirst = used;
         elen = l;
       }
@@ -450,6 +486,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
     t.a0 = __shfl_sync(kFull, t.a0, from);
     t.b0 = __shfl_sync(kFull, t.b0, from);
     t.cells = __shfl_sync(kFull, t.cells, from);
+    t.restarts = __shfl_sync(kFull, t.restarts, from);
     t.active = lane < total;
     first = nfirst;
     len = old_want;
@@ -462,6 +499,7 @@ __device__ __forceinline__ void bits_shared_run(const ExtendParams& p, int* map)
         bits_load<NB, 1>(p, L, entry, place + 32 * (lane - first));
       } else {
         F::init(L, 16 * kInitLanes - 32 * (lane - first));
+        if (over) t.restarts = __ldcg(&p.ext[t.item].status);
       }
     }
     if (!t.active) {
