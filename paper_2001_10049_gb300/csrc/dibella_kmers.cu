@@ -745,6 +745,12 @@ constexpr int kBucketSeg = 2048;    // retained occurrences held in shared memor
 constexpr int kBucketProbes = 96;
 constexpr int kBucketBlocksPerSM = 3;
 constexpr int kBucketHeld = 12;     // occurrences that a thread holds in registers (buckets up to 3,072)
+// A bucket of more than kBucketBig occurrences holds frequent codes (the codes are
+// spread evenly, their occurrences are not); it is thinned by many blocks, a part of
+// kThinPart occurrences each, before its one block counts it.
+constexpr int kBucketBig = 16384;
+constexpr int kThinPart = 8192;
+static_assert(kThinPart <= kBucketBig, "a big bucket holds the first or the last occurrence of each part that it meets");
 
 // Bits of the mixed code that number the buckets of up to n occurrences.
 int bucket_bits(unsigned long long n, int k) {
@@ -753,16 +759,25 @@ int bucket_bits(unsigned long long n, int k) {
   return b;
 }
 
+// The bucket of a key: its bits from `shift` (up to 64) on.
+__device__ __forceinline__ unsigned bucket_of(unsigned long long key, int shift) {
+  return shift < 64 ? (unsigned)(key >> shift) : 0u;
+}
+
 // starts[b] = the first occurrence of bucket b, for b = 0 .. n_buckets (the
-// occurrences are in bucket order; `shift` brings a key's bucket to bit 0).
+// occurrences are in bucket order), and thinned[b] = 0 for those below n_buckets.
 __global__ void bucket_starts_kernel(const unsigned long long* __restrict__ keys, const unsigned long long* n_ptr,
-                                     int shift, unsigned n_buckets, unsigned long long* starts) {
+                                     int shift, unsigned n_buckets, unsigned long long* starts,
+                                     unsigned long long* thinned) {
   const unsigned long long n = *n_ptr;
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i <= n; i += stride) {
-    const unsigned lo = i == 0 ? 0u : (shift < 64 ? (unsigned)(keys[i - 1] >> shift) : 0u) + 1u;
-    const unsigned hi = i == n ? n_buckets : (shift < 64 ? (unsigned)(keys[i] >> shift) : 0u);
-    for (unsigned b = lo; b <= hi; ++b) starts[b] = i;
+    const unsigned lo = i == 0 ? 0u : bucket_of(keys[i - 1], shift) + 1u;
+    const unsigned hi = i == n ? n_buckets : bucket_of(keys[i], shift);
+    for (unsigned b = lo; b <= hi; ++b) {
+      starts[b] = i;
+      if (b < n_buckets) thinned[b] = 0;
+    }
   }
 }
 
@@ -786,15 +801,106 @@ __device__ __forceinline__ unsigned bucket_scan(unsigned v, unsigned* wsum, unsi
   return before + x - v;
 }
 
+// The slot of a code (its bits below the bucket) in a table of kBucketSlots; an
+// empty one is taken with `insert`.  -1: not found in kBucketProbes slots.
+template <typename Tag>
+__device__ __forceinline__ int bucket_slot(Tag* tag, unsigned long long rest, bool insert) {
+  const Tag t = (Tag)(rest + 1);
+  unsigned s = (unsigned)((rest * 0xD6E8FEB86659FD93ull) >> 40) & (kBucketSlots - 1);
+  for (int q = 0; q < kBucketProbes; ++q) {
+    Tag c = tag[s];
+    if (c == 0 && insert) c = atomicCAS(&tag[s], (Tag)0, t);
+    if (c == t || c == 0) return (int)s;  // (c == 0: just inserted)
+    s = (s + 1) & (kBucketSlots - 1);
+  }
+  return -1;
+}
+
+// Copies the occurrences of the big buckets to `spare` (a bucket to its own place
+// there, in any order; thinned[b] gets their number), leaving out those that
+// follow mult_hi + 1 others of their code in the same part: enough are left to
+// reject the code.  A block per part.
+// Why: a bucket is counted by one block at about 0.25 G occurrences/s, so a code
+// with 7 or 69 M occurrences among 138 M (5 or 50% of the reads poly-A) held the
+// call for 30 or 300 ms, where a sort by the whole code took 14.3 or 9.4; thinned it
+// takes 7.3 or 5.7 (500 kb of poly-A: 0.74 ms, sorted 0.34, thinned 0.18).  Bound by
+// reading the keys of the big buckets; where there are none, it looks at two keys in
+// 8,192 (E. coli-sized call 8.89 ms with it, 8.87 without; the tiny set's 278.6 us, 277.1).
+template <typename Tag>
+__global__ void __launch_bounds__(kBucketThreads) thin_buckets_kernel(
+    const unsigned long long* __restrict__ keys, unsigned long long* spare, const unsigned long long* n_ptr,
+    const unsigned long long* starts, unsigned long long* thinned, int shift, int ib, int rest_bits, int mult_hi) {
+  extern __shared__ __align__(16) unsigned char bsm[];
+  Tag* tag = (Tag*)bsm;
+  unsigned* slot = (unsigned*)(tag + kBucketSlots);
+  __shared__ unsigned wsum[kBucketThreads / 32], hits[kBucketThreads / 32];
+  __shared__ unsigned long long out_at;
+  const unsigned long long n = *n_ptr, n_parts = (n + kThinPart - 1) / kThinPart;
+  const unsigned long long rmask = rest_bits == 64 ? ~0ull : (1ull << rest_bits) - 1ull;
+  auto big = [&](unsigned b) { return starts[b + 1] - starts[b] > (unsigned long long)kBucketBig; };
+  // Each thread looks at one part: whether its first or last occurrence lies in a
+  // big bucket.  Parts in a row go to blocks in a row.
+  for (unsigned long long p0 = blockIdx.x; p0 < n_parts; p0 += (unsigned long long)gridDim.x * kBucketThreads) {
+    const unsigned long long part = p0 + (unsigned long long)threadIdx.x * gridDim.x;
+    bool hit = false;
+    if (part < n_parts) {
+      const unsigned long long a = part * kThinPart, e = a + kThinPart < n ? a + kThinPart : n;
+      hit = big(bucket_of(keys[a], shift)) || big(bucket_of(keys[e - 1], shift));
+    }
+    const unsigned bal = __ballot_sync(kFullMask, hit);
+    if ((threadIdx.x & 31) == 0) hits[threadIdx.x >> 5] = bal;
+    __syncthreads();
+    for (int w = 0; w < kBucketThreads / 32; ++w) {
+      for (unsigned left = hits[w]; left != 0; left &= left - 1) {  // (uniform)
+        const unsigned long long a = (p0 + (unsigned long long)(32 * w + __ffs((int)left) - 1) * gridDim.x) * kThinPart;
+        const unsigned long long e = a + kThinPart < n ? a + kThinPart : n;
+        const unsigned b0 = bucket_of(keys[a], shift), b1 = bucket_of(keys[e - 1], shift);
+        for (int side = 0; side < 2; ++side) {
+          const unsigned b = side == 0 ? b0 : b1;
+          if ((side == 1 && b1 == b0) || !big(b)) continue;
+          const unsigned long long lo = starts[b] > a ? starts[b] : a, hi = starts[b + 1] < e ? starts[b + 1] : e;
+          for (int s = threadIdx.x; s < kBucketSlots; s += kBucketThreads) {
+            tag[s] = 0;
+            slot[s] = 0;
+          }
+          __syncthreads();
+          unsigned keep = 0;  // bit q: this thread's occurrence q (a code without a slot is kept)
+          static_assert(kThinPart <= 32 * kBucketThreads, "a part's occurrences are bits of `keep`");
+#pragma unroll 4
+          for (int q = 0; q < kThinPart / kBucketThreads; ++q) {
+            const unsigned long long i = lo + (unsigned)(q * kBucketThreads) + threadIdx.x;
+            if (i >= hi) continue;
+            const int s = bucket_slot<Tag>(tag, (keys[i] >> ib) & rmask, true);
+            if (s < 0 || (*(volatile unsigned*)&slot[s] <= (unsigned)mult_hi &&
+                          atomicAdd(&slot[s], 1u) <= (unsigned)mult_hi))
+              keep |= 1u << q;
+          }
+          unsigned all;
+          unsigned at = bucket_scan((unsigned)__popc(keep), wsum, &all);
+          if (threadIdx.x == 0) out_at = atomicAdd(&thinned[b], (unsigned long long)all);
+          __syncthreads();
+          unsigned long long* out = spare + starts[b] + out_at;
+          for (; keep != 0; keep &= keep - 1)
+            out[at++] = keys[lo + (unsigned)((__ffs((int)keep) - 1) * kBucketThreads) + threadIdx.x];
+          __syncthreads();
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // A block per bucket: count its codes, then form the occurrence pairs of the
 // retained ones (as emit_pairs_kernel does), as one-word or two-word keys.  A
 // bucket with more distinct codes than the table takes is counted in parts, by
 // the next bits of the code, halved until each part fits.  Tag: 32 bits where
-// the rest of the code fits.
+// the rest of the code fits.  A big bucket is read from `spare` (see
+// thin_buckets_kernel), and its place in `keys` is what is spare for it.
 template <typename K, typename Tag>
 __global__ void __launch_bounds__(kBucketThreads, kBucketBlocksPerSM) bucket_emit_kernel(
-    const unsigned long long* __restrict__ keys, const unsigned long long* __restrict__ info, unsigned long long* spare,
-    const unsigned long long* starts, unsigned n_buckets, int ib, int rest_bits, int mult_lo, int mult_hi, KeyLayout kl,
+    unsigned long long* all_keys, const unsigned long long* __restrict__ info, unsigned long long* all_spare,
+    const unsigned long long* starts, const unsigned long long* thinned, unsigned n_buckets, int ib, int rest_bits,
+    int mult_lo, int mult_hi, KeyLayout kl,
     K* keys_out, unsigned long long capacity, CandState* st) {
   extern __shared__ __align__(16) unsigned char bsm[];
   unsigned long long* seg_s = (unsigned long long*)bsm;
@@ -810,8 +916,16 @@ __global__ void __launch_bounds__(kBucketThreads, kBucketBlocksPerSM) bucket_emi
   const unsigned long long rmask = rest_bits == 64 ? ~0ull : (1ull << rest_bits) - 1ull;
   unsigned long long kept_codes = 0;
   for (unsigned b = blockIdx.x; b < n_buckets; b += gridDim.x) {
-    const unsigned long long lo = starts[b], hi = starts[b + 1];
+    const unsigned long long lo = starts[b];
+    unsigned long long hi = starts[b + 1];
     if (lo == hi) continue;  // (uniform)
+    const unsigned long long* keys = all_keys;
+    unsigned long long* spare = all_spare;
+    if (hi - lo > (unsigned long long)kBucketBig) {
+      hi = lo + thinned[b];
+      keys = all_spare;
+      spare = all_keys;
+    }
     int j = 0;
     for (unsigned long long part = 0;;) {
       // ---- count the codes whose highest j bits of the rest are `part` ----
@@ -821,21 +935,10 @@ __global__ void __launch_bounds__(kBucketThreads, kBucketBlocksPerSM) bucket_emi
       }
       if (threadIdx.x == 0) overflow = 0;
       __syncthreads();
-      auto find = [&](unsigned long long rest, bool insert) -> int {
-        const Tag t = (Tag)(rest + 1);
-        unsigned s = (unsigned)((rest * 0xD6E8FEB86659FD93ull) >> 40) & (kBucketSlots - 1);
-        for (int q = 0; q < kBucketProbes; ++q) {
-          Tag c = tag[s];
-          if (c == 0 && insert) c = atomicCAS(&tag[s], (Tag)0, t);
-          if (c == t || c == 0) return (int)s;  // (c == 0: just inserted)
-          s = (s + 1) & (kBucketSlots - 1);
-        }
-        return -1;
-      };
       const bool held = j == 0 && hi - lo <= (unsigned long long)(kBucketHeld * kBucketThreads);
       unsigned long long mine[kBucketHeld];  // held: this thread's keys, then (in the low bits) their slots
       auto count = [&](unsigned long long rest) -> int {
-        const int s = find(rest, true);
+        const int s = bucket_slot<Tag>(tag, rest, true);
         if (s < 0)
           overflow = 1;
         else if (slot[s] <= (unsigned)mult_hi)  // (one too many is enough: no pile-up on a frequent code)
@@ -916,7 +1019,7 @@ __global__ void __launch_bounds__(kBucketThreads, kBucketBlocksPerSM) bucket_emi
           for (unsigned long long i = lo + threadIdx.x; i < hi; i += kBucketThreads) {
             const unsigned long long key = keys[i], rest = (key >> ib) & rmask;
             if (j > 0 && (rest >> (rest_bits - j)) != part) continue;
-            const int s = find(rest, false);
+            const int s = bucket_slot<Tag>(tag, rest, false);
             if (s < 0 || slot[s] == 0) continue;
             const unsigned v = atomicAdd(&slot[s], 1u);
             seg[(v >> 12) + (v & 63u)] = info[key & imask];
@@ -968,7 +1071,16 @@ __global__ void __launch_bounds__(kBucketThreads, kBucketBlocksPerSM) bucket_emi
       if (j == 0) break;
     }
   }
-  kept_codes = warp_atomic_add(&st->retained, kept_codes);
+  warp_atomic_add(&st->retained, kept_codes);
+  __syncthreads();
+  if (threadIdx.x == 0) {  // the block that ends last caps the keys, as cap_keys_kernel does
+    __threadfence();
+    if (atomicAdd(&st->ticket, 1u) == gridDim.x - 1) {
+      const unsigned long long pairs = atomicAdd(&st->occ_pairs, 0ull);
+      st->n_keys = pairs < capacity ? pairs : capacity;
+      st->ticket = 0;
+    }
+  }
 }
 
 template <typename Tag>
@@ -993,28 +1105,33 @@ cudaError_t count_in_buckets(unsigned long long* buf0, unsigned long long* buf1,
     buf1 = tmp;
   }
   const unsigned n_buckets = 1u << bits;
-  unsigned long long* starts = hoff;  // the last pass has read its offsets; n_buckets + 1 <= 256 tiles entries
-  bucket_starts_kernel<<<sms * 8, 256, 0, st>>>(buf0, n_ptr, ib + rest_bits, n_buckets, starts);
+  // the last pass has read its offsets; 2 n_buckets + 1 <= 256 tiles entries
+  unsigned long long* starts = hoff;
+  unsigned long long* thinned = starts + n_buckets + 1;
+  bucket_starts_kernel<<<sms * 8, 256, 0, st>>>(buf0, n_ptr, ib + rest_bits, n_buckets, starts, thinned);
   // 64 KB of shared memory a block, 80 with 64-bit tags
   const unsigned resident = (unsigned)(sms * (rest_bits < 32 ? kBucketBlocksPerSM : 2));
   const unsigned blocks = n_buckets < resident ? n_buckets : resident;
-  cudaError_t e;
-  if (rest_bits < 32) {
-    const auto fn = bucket_emit_kernel<K, unsigned int>;
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bucket_smem<unsigned int>())) !=
+  const auto launch = [&](auto tag) -> cudaError_t {
+    using Tag = decltype(tag);
+    cudaError_t e;
+    if (n_max > (unsigned long long)kBucketBig) {
+      const auto fn = thin_buckets_kernel<Tag>;
+      const int smem = kBucketSlots * (int)(sizeof(Tag) + 4);
+      if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+      const unsigned long long parts = (n_max + kThinPart - 1) / kThinPart, fit = 4ull * (unsigned)sms;
+      fn<<<(unsigned)(parts < fit ? parts : fit), kBucketThreads, smem, st>>>(buf0, buf1, n_ptr, starts, thinned,
+                                                                              ib + rest_bits, ib, rest_bits, mult_hi);
+    }
+    const auto fn = bucket_emit_kernel<K, Tag>;
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bucket_smem<Tag>())) !=
         cudaSuccess)
       return e;
-    fn<<<blocks, kBucketThreads, bucket_smem<unsigned int>(), st>>>(buf0, info, buf1, starts, n_buckets, ib, rest_bits,
-                                                                    mult_lo, mult_hi, kl, keys_out, capacity, state);
-  } else {
-    const auto fn = bucket_emit_kernel<K, unsigned long long>;
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)bucket_smem<unsigned long long>())) != cudaSuccess)
-      return e;
-    fn<<<blocks, kBucketThreads, bucket_smem<unsigned long long>(), st>>>(
-        buf0, info, buf1, starts, n_buckets, ib, rest_bits, mult_lo, mult_hi, kl, keys_out, capacity, state);
-  }
-  return cudaGetLastError();
+    fn<<<blocks, kBucketThreads, bucket_smem<Tag>(), st>>>(buf0, info, buf1, starts, thinned, n_buckets, ib, rest_bits,
+                                                           mult_lo, mult_hi, kl, keys_out, capacity, state);
+    return cudaGetLastError();
+  };
+  return rest_bits < 32 ? launch(0u) : launch(0ull);
 }
 
 // The partitioned count: one pass per hash part of the canonical codes.  Every
@@ -1418,7 +1535,6 @@ int dibella_candidate_pairs_parts(const uint32_t* packed_words, const int64_t* r
                            (unsigned long long*)(ws + L.pk0), L.pairs, hist, hoff, part, state, sms, st);
     if (e != cudaSuccess) return DIBELLA_ECUDA;
   }
-  cap_keys_kernel<<<1, 1, 0, st>>>(state, L.pairs);
   const int gap = min_seed_gap > 0 ? min_seed_gap : k;
   if (wide) {
     Key2* src = (Key2*)(ws + L.pk0);
@@ -1537,8 +1653,8 @@ int dibella_candidate_pairs(const uint32_t* packed_words, const int64_t* read_wo
     allocate_kernel<<<sms * 8, 256, 0, st>>>(t, L.slots, mult_lo, mult_hi, retained, state);
     kmer_walk_kernel<true><<<walk_blocks, 256, 0, st>>>(sr, t, inst, L.inst, mult_lo, mult_hi, state);
     emit_pairs_kernel<<<sms * 8, 256, 0, st>>>(t, retained, inst, L.inst, kl, pk0, L.pairs, state);
+    cap_keys_kernel<<<1, 1, 0, st>>>(state, L.pairs);
   }
-  cap_keys_kernel<<<1, 1, 0, st>>>(state, L.pairs);
   // Radix sort by the whole key (read_a, read_b, pos_a, pos_b, strand).
   const int key_bits = kl.sh_ra + rbits;
   const int passes = (key_bits + 7) / 8;
