@@ -736,7 +736,7 @@ __global__ void extract_kernel(StoreRef sr, const unsigned long long* off, int i
 // The occurrences are sorted only by the highest bucket_bits of their mixed
 // code; a bucket of about kBucketMean occurrences is then counted in a block's
 // shared memory.  Sorting all 34 bits of a 17-mer takes 5 passes over the keys
-// (24 bytes each per key), this takes 2 and one read of each bucket, from which
+// (24 bytes each per key), this takes 2 (3 from 201 M occurrences on) and one read of each bucket, from which
 // the pairs are emitted too, with one global atomic per bucket and counter.
 constexpr int kBucketMean = 2048;
 constexpr int kBucketThreads = 256;
@@ -752,10 +752,16 @@ constexpr int kBucketBig = 16384;
 constexpr int kThinPart = 8192;
 static_assert(kThinPart <= kBucketBig, "a big bucket holds the first or the last occurrence of each part that it meets");
 
-// Bits of the mixed code that number the buckets of up to n occurrences.
-int bucket_bits(unsigned long long n, int k) {
+// Bits of the mixed code that number the buckets of up to n_max occurrences, of
+// which n_mean are expected: two digits while the buckets then fit the threads'
+// registers (201 M occurrences), else three.  With two digits beyond that the
+// codes outgrow the table, and a bucket is read again for each half and quarter: a
+// pass over 200 M occurrences takes 13.9 ms, over 230 M 20.3 (18.6 with three digits),
+// 300 M 30.1 (22.7), 515 M 68.7 (41.0; 76.4 in one sort by the whole code).
+int bucket_bits(unsigned long long n_max, unsigned long long n_mean, int k) {
+  const int most = (n_mean >> 16) > (unsigned long long)(kBucketHeld * kBucketThreads) ? 24 : 16;
   int b = 0;
-  while (b < 16 && b < 2 * k && (n >> b) > (unsigned long long)kBucketMean) ++b;
+  while (b < most && b < 2 * k && (n_max >> b) > (unsigned long long)kBucketMean) ++b;
   return b;
 }
 
@@ -959,11 +965,18 @@ __global__ void __launch_bounds__(kBucketThreads, kBucketBlocksPerSM) bucket_emi
           }
         }
       } else {
-#pragma unroll 4
-        for (unsigned long long i = lo + threadIdx.x; i < hi; i += kBucketThreads) {
-          const unsigned long long rest = (keys[i] >> ib) & rmask;
-          if (j > 0 && (rest >> (rest_bits - j)) != part) continue;
-          count(rest);
+        // (a table that is full is left at once: every further code would probe it in vain)
+        constexpr int kU = 4;
+        for (unsigned long long i0 = lo + threadIdx.x; i0 < hi && *(volatile int*)&overflow == 0;
+             i0 += kU * kBucketThreads) {
+          unsigned long long key[kU];
+#pragma unroll
+          for (int u = 0; u < kU; ++u) key[u] = i0 + u * kBucketThreads < hi ? keys[i0 + u * kBucketThreads] : 0ull;
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const unsigned long long rest = (key[u] >> ib) & rmask;
+            if (i0 + u * kBucketThreads < hi && (j == 0 || (rest >> (rest_bits - j)) == part)) count(rest);
+          }
         }
       }
       __syncthreads();
@@ -1088,15 +1101,15 @@ constexpr size_t bucket_smem() {
   return (size_t)kBucketSeg * 8 + (size_t)kBucketSlots * (sizeof(Tag) + 8);
 }
 
-// Orders n_ptr occurrences (at most n_max; in buf0, buf1 spare) by bucket and emits
+// Orders n_ptr occurrences (at most n_max, n_mean expected; in buf0, buf1 spare) by bucket and emits
 // their pairs.  Keys: mixed code << ib | index.
 template <typename K>
 cudaError_t count_in_buckets(unsigned long long* buf0, unsigned long long* buf1, const unsigned long long* info,
-                             const unsigned long long* n_ptr, unsigned long long n_max, int k, int ib, int mult_lo,
-                             int mult_hi, const KeyLayout& kl, K* keys_out, unsigned long long capacity,
+                             const unsigned long long* n_ptr, unsigned long long n_max, unsigned long long n_mean,
+                             int k, int ib, int mult_lo, int mult_hi, const KeyLayout& kl, K* keys_out, unsigned long long capacity,
                              unsigned int* hist, unsigned long long* hoff, unsigned long long* part, CandState* state,
                              int sms, cudaStream_t st) {
-  const int bits = bucket_bits(n_max, k), rest_bits = 2 * k - bits;
+  const int bits = bucket_bits(n_max, n_mean, k), rest_bits = 2 * k - bits;
   const unsigned long long tiles = (n_max + KeyOps<unsigned long long>::kTile - 1) / KeyOps<unsigned long long>::kTile;
   for (int j = 0; j < (bits + 7) / 8; ++j) {
     radix_pass(buf0, buf1, n_ptr, ib + rest_bits + 8 * j, hist, hoff, tiles, part, state, sms, st);
@@ -1522,16 +1535,17 @@ int dibella_candidate_pairs_parts(const uint32_t* packed_words, const int64_t* r
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms <= 0) sms = 1;
   StoreRef sr{packed_words, read_word_offsets, read_lengths, (long long)n_reads, k};
+  const unsigned long long n_mean = (unsigned long long)n_bases / (unsigned)n_parts;
   for (int p = 0; p < n_parts && n_reads > 0; ++p) {
     pass_begin_kernel<<<1, 1, 0, st>>>(state);
     extract_part_kernel<<<sms * 16, 256, 0, st>>>(sr, (unsigned)p, (unsigned)n_parts, ib, L.pass_cap, ok0, info,
                                                   state);
     pass_end_kernel<<<1, 1, 0, st>>>(state, L.pass_cap);
     if (wide)
-      e = count_in_buckets(ok0, ok1, info, &state->pass_held, L.pass_cap, k, ib, mult_lo, mult_hi, kl,
+      e = count_in_buckets(ok0, ok1, info, &state->pass_held, L.pass_cap, n_mean, k, ib, mult_lo, mult_hi, kl,
                            (Key2*)(ws + L.pk0), L.pairs, hist, hoff, part, state, sms, st);
     else
-      e = count_in_buckets(ok0, ok1, info, &state->pass_held, L.pass_cap, k, ib, mult_lo, mult_hi, kl,
+      e = count_in_buckets(ok0, ok1, info, &state->pass_held, L.pass_cap, n_mean, k, ib, mult_lo, mult_hi, kl,
                            (unsigned long long*)(ws + L.pk0), L.pairs, hist, hoff, part, state, sms, st);
     if (e != cudaSuccess) return DIBELLA_ECUDA;
   }
@@ -1645,7 +1659,7 @@ int dibella_candidate_pairs(const uint32_t* packed_words, const int64_t* read_wo
     const dim3 grid((unsigned)(need < walk_blocks ? need : walk_blocks),
                     (unsigned)(share < 1 ? 1 : (share > 64 ? 64 : share)));
     extract_kernel<<<grid, 256, 0, st>>>(sr, occ_off, ib, L.inst, ok0, info);
-    if ((e = count_in_buckets(ok0, ok1, info, &state->instances, L.inst, k, ib, mult_lo, mult_hi, kl, pk0, L.pairs,
+    if ((e = count_in_buckets(ok0, ok1, info, &state->instances, L.inst, L.inst, k, ib, mult_lo, mult_hi, kl, pk0, L.pairs,
                               hist, hoff, part, state, sms, st)) != cudaSuccess)
       return DIBELLA_ECUDA;
   } else if (n_reads > 0) {

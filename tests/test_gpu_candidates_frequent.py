@@ -55,8 +55,7 @@ def test_one_bucket_holds_everything():
 
 def test_one_code_is_not_one_blocks_work():
     """20 Mb of poly-A take no longer than a few times 20 Mb of random bases
-    (half of 138 M occurrences being one code, counted by one block, made it 300 ms
-    where there are 8 without)."""
+    (42 ms against 1.4 when one block counted them alone)."""
     import torch
     import paper_2001_10049_gb300 as dib
     rng = np.random.default_rng(5)
