@@ -333,11 +333,12 @@ def mode_tune(args):
     """Uneven batch (log-uniform 500 bp - 100 kb reads, per-read error 5-35%,
     X = 50; or another workload and X): the schedule the autotuner picks on an
     independent draw of the same workload (generator seed + 100), so the tuned
-    schedule is judged on data it was not tuned on, against the library's
-    default schedule and against a naive fixed one (one length bucket, every
-    extension to the warp-per-extension form).  (A 10% sample of the batch
-    itself misled the tuner: with a tenth of the extensions per warp, the
-    longest extensions dominate its timings.)"""
+    schedule is judged on data it was not tuned on, against a call without a
+    schedule (`fixed`: for these scores the bit-sliced form up to X = 59), against
+    the default schedule in the int16 forms, and against a naive fixed one (one
+    length bucket, every extension to the warp-per-extension form).  (A 10%
+    sample of the batch itself misled the tuner: with a tenth of the extensions
+    per warp, the longest extensions dominate its timings.)"""
     import torch
     import paper_2001_10049_gb300 as dib
     dev = torch.device("cuda", 0)
@@ -355,9 +356,12 @@ def mode_tune(args):
     naive_d = fixed.as_dict()
     naive_d.update(narrow_max_xdrop=-1, n_buckets=1, bucket_bounds=[], mid_band_cap=0)
     naive = dib.Schedule.from_dict(naive_d)
+    # the default but for narrow_unroll, where 16 means what 0 does: followed as given, in the int16 forms
+    int16 = dib.Schedule.from_dict(dict(fixed.as_dict(), narrow_unroll=16))
     with ClockSampler(0) as clocks:
-        fixed_ms = _time_direct(torch, al, n, sc, stream, fixed, args.steps)
+        fixed_ms = _time_direct(torch, al, n, sc, stream, None, args.steps)
         c_fixed = dib.dibella_batch_counters(al.workspace, stream=stream)
+        int16_ms = _time_direct(torch, al, n, sc, stream, int16, args.steps)
         naive_ms = _time_direct(torch, al, n, sc, stream, naive, args.steps)
         tw = workloads.generate(wname, seed=workloads.CONFIGS[wname]["seed"] + 100)
         tstore = dib.ReadStore.from_ascii(tw.reads, tw.offsets, device=dev)
@@ -380,7 +384,7 @@ def mode_tune(args):
         "config": {"workload": wname, "reads": int(w.n_reads), "candidate_pairs": n_cand, "seed_records": n,
                    "extensions": 2 * n, "xdrop": X, "scoring": "+1/-1/-1", "k": K, "steps": args.steps,
                    "l2": "flushed (256 MiB write) before every timed batch"},
-        "fixed": {"schedule": fixed.as_dict(), "ms": fixed_ms, "pairs_per_s": n_cand / (fixed_ms * 1e-3),
+        "fixed": {"schedule": None, "ms": fixed_ms, "pairs_per_s": n_cand / (fixed_ms * 1e-3),
                   "gcups": cells / (fixed_ms * 1e-3) / 1e9, "counters": c_fixed},
         "tuned": {"schedule": best.as_dict(), "ms": tuned_ms, "pairs_per_s": n_cand / (tuned_ms * 1e-3),
                   "gcups": cells / (tuned_ms * 1e-3) / 1e9, "counters": c_tuned, "tuning_batch_ms": best_ms,
@@ -388,6 +392,7 @@ def mode_tune(args):
                   "tuned_on": "an independent draw of %s (generator seed %d): %d candidate pairs, "
                               "%d seed records" % (wname, workloads.CONFIGS[wname]["seed"] + 100,
                                                    len(workloads.pair_groups(tw.pairs)) - 1, len(tw.pairs))},
+        "int16_default": {"schedule": int16.as_dict(), "ms": int16_ms, "pairs_per_s": n_cand / (int16_ms * 1e-3)},
         "naive": {"schedule": naive.as_dict(), "ms": naive_ms, "pairs_per_s": n_cand / (naive_ms * 1e-3)},
         "speedup_tuned_vs_fixed": fixed_ms / tuned_ms,
         "speedup_tuned_vs_naive": naive_ms / tuned_ms,

@@ -140,9 +140,10 @@ int dibella_pack_reads(const char* ascii, const int64_t* ascii_offsets, int64_t 
  * per extension with an 8192-cell band in shared memory (the CTA form), and
  * beyond that by a warp whose band lives in the workspace (sized by
  * max_read_len: it cannot overflow).
- * When a call passes no schedule (and the default is the built-in one), match
- * 1, mismatch -1, gap -1 and 1 <= xdrop <= 59 take none of these but the
- * bit-sliced form: 32 cells of a lane in one register per score bit, 1 to 32
+ * When a call passes no schedule and the default is the built-in one, or passes
+ * the built-in one (what dibella_get_default_schedule returns until another is
+ * set), match 1, mismatch -1, gap -1 and 1 <= xdrop <= 59 take none of these but
+ * the bit-sliced form: 32 cells of a lane in one register per score bit, 1 to 32
  * lanes per extension by the width of its band (a whole warp with 2 and 4
  * words per lane for bands up to 4,096 cells, then the CTA form and the band in
  * the workspace as above).
@@ -152,8 +153,8 @@ int dibella_pack_reads(const char* ascii, const int64_t* ascii_offsets, int64_t 
  * go entirely to the wide form (they would wait on one lane's longest
  * extension), and for xdrop > 10 keys above 20000 (above 5000 in batches
  * with fewer than 7 extensions per lane) go to the wide form (a narrow lane
- * would otherwise hold up the escalations behind its long extension); an
- * explicit schedule is followed as given.  Work is ordered by
+ * would otherwise hold up the escalations behind its long extension); any
+ * other explicit schedule is followed as given.  Work is ordered by
  * n_buckets length buckets (longest first); bucket b holds keys below
  * bucket_bounds[b] (ascending), the last bucket everything else. */
 #define DIBELLA_MAX_BUCKETS 8
@@ -464,8 +465,9 @@ int dibella_xdrop_traceback(const uint32_t* packed_words, const int64_t* read_wo
  * dibella_xdrop_batch; results hold the last run's output.  Synchronises
  * `stream`; refused (EINVAL) while `stream` is capturing.  *best_ms_out and
  * *n_tried_out (either may be NULL) receive the winner's time and the number
- * of schedules timed.  (Every one of them is an explicit schedule: where the
- * bit-sliced form applies, a call without a schedule is faster.)
+ * of schedules timed.  The built-in schedule is among them: where the
+ * bit-sliced form applies, it runs in that form and the others do not, so that
+ * the search returns it unless one of them is faster.
  * The paper has no tuner; its Sec. 9 names the cost
  * differences (read length, X-drop early exit) this one adapts to. */
 int dibella_autotune(const uint32_t* packed_words, const int64_t* read_word_offsets,
