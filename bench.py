@@ -279,6 +279,15 @@ def workload_config(w, n_cand, n_seeds, xdrops, note=""):
             "xdrop": list(xdrops), "scoring": "+1/-1/-1", "k": K, "l2": L2_NOTE}
 
 
+BITS_FORM, BITS_MAX_X = "bit-sliced form, shared lanes", 59
+
+
+def first_form_names(built_in_schedule, xdrops):
+    """The form of a batch's first extension launch, by X (unit scores; with the
+    built-in schedule, or none, the bit-sliced one up to its largest X)."""
+    return {X: BITS_FORM if built_in_schedule and 1 <= X <= BITS_MAX_X else "narrow form" for X in xdrops}
+
+
 def run_reference(args, world, rank):
     if rank != 0:
         return
@@ -826,6 +835,7 @@ def main():
         shard_info = {"cost_keys": [int(t) for t in totals], "max_over_mean": float(totals.max() / totals.mean())}
     n_seeds = len(pairs)
     sched = None
+    built_in = dib.dibella_get_default_schedule().as_dict()
     if args.default_schedule:
         d = dib.dibella_get_default_schedule().as_dict()
         d.update(json.loads(args.default_schedule))
@@ -834,6 +844,7 @@ def main():
         d = dib.dibella_get_default_schedule().as_dict()
         d.update(json.loads(args.schedule))
         sched = dib.Schedule.from_dict(d)
+    first_form = first_form_names((sched or dib.dibella_get_default_schedule()).as_dict() == built_in, XD)
     n_cand = len(workloads.pair_groups(pairs)) - 1
     store = dib.ReadStore.from_ascii(w.reads, w.offsets, device=dev)
     al = dib.Aligner(store, n_seeds, k=K, device=dev)
@@ -932,7 +943,8 @@ def main():
                 continue
             wc = wc[wc[:, 1] > 0].astype(np.int64)
             fin = wc[:, 1] - wc[:, 0].min()
-            balance[str(X)][name] = {"warps": int(len(wc)), "span_ms": float(fin.max() / 1e6),
+            form = first_form[X] if which == 1 else name
+            balance[str(X)][form] = {"warps": int(len(wc)), "span_ms": float(fin.max() / 1e6),
                                      "mean_finish_ms": float(fin.mean() / 1e6),
                                      "max_over_mean": float(fin.max() / max(fin.mean(), 1.0)),
                                      "p50_finish_ms": float(np.percentile(fin, 50) / 1e6)}
@@ -991,9 +1003,8 @@ def main():
     for X in XD:
         phase[X] = np.concatenate([phase[X][:1], [phase[X][1] + phase[X][2]], phase[X][3:]])
     batch_ms = {X: float(np.mean([ms for (x, ms, _) in log if x == X])) for X in XD}
-    # without a schedule every extension runs in the bit-sliced form, whose one launch stands as the narrow form's
-    first_form = "narrow form" if sched is not None else "bit-sliced form, shared lanes"
-    launch_cells = {X: {first_form: (1, counters[X]["cells_narrow"]),
+    # in the bit-sliced form the one launch of every extension stands as the narrow form's
+    launch_cells = {X: {first_form[X]: (1, counters[X]["cells_narrow"]),
                         "wide form, first launch": (2, counters[X]["cells_wide"] - counters[X]["cells_wide_esc"]
                                                      - counters[X]["cells_ladder"]),
                         "mid form on the narrow escalations": (3, counters[X]["cells_mid"]),
@@ -1049,9 +1060,10 @@ def main():
                      "peak_source": "%d SMs x %d INT32 lanes x %.0f MHz (%s sm_max_mhz)"
                                     % (sm_count, INT32_LANES_PER_SM, pk.get("sm_max_mhz", 2070.0), pk_kind),
                      "ops_per_cell": OPS_PER_CELL,
-                     "ops_note": "8 per cell is the convention of a cell-by-cell DP; the bit-sliced form issues about "
-                                 "3 lane instructions a cell of its windows (32 cells to a logic instruction), so the "
-                                 "fractions compare it with such a DP; its integer pipe is 85 to 92% busy",
+                     "ops_note": "8 per cell is the convention of a cell-by-cell DP"
+                                 + ("; the bit-sliced form issues about 3 lane instructions a cell of its windows (32 "
+                                    "cells to a logic instruction), so the fractions compare it with such a DP and are "
+                                    "not a utilisation" if domName == BITS_FORM else ""),
                      "peak_measured": cell_peak, "frac_measured": achieved / cell_peak,
                      "peak_measured_class": "int32 DP cell, 8 ops (compare, select, add; max, add; max; "
                                             "compare, select), full grid of independent chains",
