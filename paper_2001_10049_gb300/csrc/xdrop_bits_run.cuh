@@ -175,13 +175,16 @@ __device__ __forceinline__ void bits_load(const ExtendParams& p, BitLane<NB, W>&
 template <int NB, int W>
 __device__ __forceinline__ void bits_settle(BitLane<NB, W>& L, BitTask& t, int lane, int first, int len,
                                             const GroupMasks& gm) {
-  uint32_t s = L.cells;  // inclusive scan within the group
+  // Inclusive scan within the group, in 64 bits: a layout lasts as long as the band
+  // keeps its place, and 2^25 antidiagonals of a steady band are beyond 32 bits in
+  // the group (in a lane they stay below: 32 W cells each, W up to 4).
+  unsigned long long s = L.cells;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t v = __shfl_up_sync(kFull, s, o);
+    const unsigned long long v = __shfl_up_sync(kFull, s, o);
     if (lane - o >= first) s += v;
   }
-  t.cells += __shfl_sync(kFull, s, first + len - 1);
+  t.cells += (long long)__shfl_sync(kFull, s, first + len - 1);
   L.cells = 0;
   int lo, hi;
   group_ends<W>(L.imp, lane, first, gm.grp, lo, hi);
