@@ -432,10 +432,13 @@ int dibella_traceback_workspace_bytes(int64_t n_lanes, int32_t max_read_len, int
  * DIBELLA_RES_BAND_OVERFLOW and zero fields).  Asynchronous on `stream`
  * (a cudaStream_t); allocates nothing.  A warp per seed (n_lanes warps,
  * each with one workspace slot, taking seeds t = w, w + n_lanes, ...)
- * re-runs both extensions with the band across its lanes, then one lane walks
- * back: meant for the seeds whose edits are wanted (accepted overlaps).
+ * re-runs both extensions with the band across its lanes, then walks back:
+ * meant for the seeds whose edits are wanted (accepted overlaps).  With unit
+ * scores (1, -1, -1) and 1 <= xdrop <= 59 all lanes walk, both extensions at
+ * once where they fit; else, and for bands beyond 990 cells, one lane does.
  * Sizing: a warp walking one seed is latency bound, so give it occupancy:
- * 24 warps per SM (3,648 on 152 SMs; 80 registers per thread) traced twice
+ * 16 warps per SM (2,432 on 152 SMs) are resident with unit scores, and slots
+ * beyond them are not used; the general form holds 24, which traced twice
  * as many seeds per second as 8; moves_words must hold, per extension, 3 words per antidiagonal up
  * to the best one plus 2 bits per evaluated cell, about (m + n) x (3 + band /
  * 16) words for an m x n extension (2^18 words cover a 30 kb overlap at a

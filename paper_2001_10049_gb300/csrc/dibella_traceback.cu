@@ -26,10 +26,10 @@
 // together: each holds the move words of one or two of the next 32
 // antidiagonals, and a run of diagonal steps is one look-up.  Bands beyond 990
 // cells take the general form above.
-// 2,000 accepted overlaps of E. coli-sized reads at X = 25 take 16.0 to 19.7 ms
-// (the general form, bound by its rows in memory and one lane's walk, 52 to 73):
-// now the longest overlap alone (69,700 antidiagonals, 14.8 ms, about a third
-// of it the walk), which is a serial chain.
+// 2,000 accepted overlaps of E. coli-sized reads at X = 25 take 13.5 to 18.2 ms (the
+// general form, bound by its rows in memory and one lane's walk, 50 to 73), by the
+// longest overlap among them: a serial chain of some 70,000 antidiagonals, about a
+// third of its time the walk.
 
 #include <cuda_runtime.h>
 

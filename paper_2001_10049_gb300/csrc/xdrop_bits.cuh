@@ -22,7 +22,7 @@
 //
 // How cells are laid out.  Bit t of plane k of a lane's word w is bit k of one
 // cell, so one 3-input logic instruction works on 32 cells of a lane: about
-// 10 NB + 8 instructions for 32 cells and lane, where the packed int16 form
+// 10 NB + 8 logic operations for 32 cells and lane, where the packed int16 form
 // takes 9 for one cell and lane.  A group of G lanes with W words each holds a
 // window of 32 G W consecutive cells of one extension.  The window moves up by
 // one cell on every second antidiagonal (even steps "E" move it, odd steps "O"
@@ -46,7 +46,8 @@
 // What bounds it: the integer pipe.  An antidiagonal of a warp (5 planes, one word
 // a lane) is about 97 instructions, 79 of them on that pipe at one per two cycles a
 // scheduler; two warps a scheduler keep the pipe 85 to 92% busy (counters at X = 7,
-// 25 and 50).  Memory traffic is one word of bases per lane and 32 antidiagonals.
+// 25 and 50).  Memory traffic is at most four words of bases per lane and 32
+// antidiagonals.
 // Carrying r1 into the comparison with X instead of selecting X - r1, leaving the
 // validity planes out of loops that stay inside the matrix, and one shift for the
 // mask below the highest bit took it there from 107 and 89 (E. coli-sized batches

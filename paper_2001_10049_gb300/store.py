@@ -157,8 +157,10 @@ class Aligner:
         """The seeds' results and the run-length encoded columns of their best
         alignments (dibella_xdrop_traceback; synchronous): (results,
         ops[n, ops_per_seed] uint32, n_ops[n] int32).  Scratch: n_lanes warp
-        slots (default 24 per SM, where one warp per seed is no longer latency
-        bound) of 3 x (longest read + 2) int32 plus moves_words words."""
+        slots (default 24 per SM, what is resident in the general form; with unit
+        scores and X from 1 to 59 at most 16 per SM are used, and passing that
+        many saves a third of the scratch) of 3 x (longest read + 2) int32 plus
+        moves_words words."""
         from . import RESULT_DTYPE, Scoring, dibella_traceback_workspace_bytes, dibella_xdrop_traceback
         torch = _torch()
         s = scoring if isinstance(scoring, Scoring) else Scoring(*scoring)
